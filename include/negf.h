@@ -73,12 +73,14 @@ typedef enum {
                                    the chunk of points that was being solved                */
 
 /* Precision forms.  The mixed forms run every block GEMM on the tensor cores: each row of
- * op(A) and column of op(B) is scaled by a power of two and rounded once to a fixed-point value
- * of 39, 47 or 55 bits below twice the line maximum (the tiers are named 40, 48 and 56 bits),
- * cut into exact BF16 slices whose products are summed exactly in FP32 groups; storage,
- * pivoting, norms and reductions stay FP64.  A product's error is about
- * 2^-bits x K x max|row of A| x max|column of B|.  Issued tensor work per complex product: 15
- * (40 bits), 21 (48 bits) or 28 (56 bits) slice products for blocks up to 512 x 512. */
+ * op(A) and column of op(B) is scaled by a power of two and rounded once to fixed point (the
+ * tiers are named 40, 48 and 56 bits), and the fixed-point product is formed exactly from BF16
+ * operands; storage, pivoting, norms and reductions stay FP64.  Calls of 12 points (batch items)
+ * or more form it modulo 10-14 small integers (residue products): a product's error is about
+ * 2^-(bits + 2) x |row of A| x |column of B| (2-norms), that of an FP64 product in the 56-bit
+ * tier, and a complex product issues 20 (40 bits), 24 (48 bits) or 28 (56 bits) real products at
+ * 257-400 contracted terms.  Calls of fewer points cut the values into BF16 slices: the error is
+ * about 2^-bits x K x max|row of A| x max|column of B|, for 60, 84 or 112 real products. */
 typedef enum {
   NEGF_PREC_FP64 = 0,     /* every block operation in FP64 on the CUDA cores (reference form) */
   NEGF_PREC_MIXED = 1,    /* tensor cores, 48-bit operand values (the default mixed form)     */
@@ -345,8 +347,8 @@ negf_status negf_atoms_to_orbitals(int32_t n_slabs, int32_t block, int32_t orbit
  * 2 = conjugate transpose; op(A) is M x K, op(B) is K x N; strides are in complex elements
  * between batch items (0 = the same matrix for every item; C needs a nonzero stride when
  * n_batch > 1).  `precision` is any negf_precision.  FP64 form: CUDA cores.  Mixed forms:
- * tensor cores with exact split-BF16 slices of 40-, 48- or 56-bit values (error about
- * 2^-bits x K relative to max|A| max|B| per row and column), exact for K <= 524288
+ * tensor cores with fixed-point values of 40, 48 or 56 bits (error about 2^-bits x K relative
+ * to max|A| max|B| per row and column, or less: see negf_precision) for K <= 524288
  * (40 bits), 393216 (48 bits) or 98304 (56 bits): a longer contraction returns
  * NEGF_ERR_UNSUPPORTED (and a workspace size of 0) rather than losing accuracy.  The block
  * inverse (and so every sweep entry point) takes
@@ -396,8 +398,9 @@ negf_status negf_zinv_batched_noalloc(int32_t n_batch, int32_t n, double* M, dou
                                       int32_t* status, void* stream);
 
 /* ---- tensor-core GEMM configuration (autotuning) ----------------------------------------
- * The mixed-precision GEMM has negf_tc_config_count() kernel configurations, differing only in
- * speed: configuration c uses the kernel shape c / 2 of
+ * The mixed-precision GEMM of calls of fewer than 12 points or batch items (digit slices) has
+ * negf_tc_config_count() kernel configurations, differing only in speed (that of larger calls
+ * picks its tile by the product's size): configuration c uses the kernel shape c / 2 of
  *   (6 stages, 1 CTA, 1), (6, 1, 2), (6, 1, 3), (8 stages, CTA pair, 1), (8, 2, 2), (8, 2, 4),
  *   (3, 1, 1, 2 K chunks per stage), (4, 2, 1, 2 K chunks per stage),
  *   (2, 1, 1, 3 K chunks per stage), (2, 2, 1, 4 K chunks per stage),
@@ -417,7 +420,7 @@ int32_t negf_tc_config_get(void);
 /* ---- accounting ----------------------------------------------------------------------------
  * Instrumentation for benchmarks, not part of the method.  negf_launch_count() is the number
  * of kernels this library has launched since it was loaded.  With profiling on, every launch of
- * the tensor-core GEMM kernel (kind 0), of its operand slicing (kind 1) and every Gauss-Jordan
+ * the tensor-core GEMM kernel (kind 0), of its operand slicing or residues (kind 1) and every Gauss-Jordan
  * elimination of a block inverse inside the sweeps (kind 2: the FP32 start of the mixed form or
  * the whole FP64 inverse, without the Newton-Schulz products, which count as kinds 0 and 1) and
  * every launch of its panel-elimination kernel (kind 3, a part of kind 2) is
@@ -430,7 +433,7 @@ negf_status negf_profile_read(int32_t kind, long long* launches, double* total_m
 /* Flops of kind 0 since the last reset, counted on the device for the batch items that ran
  * (items masked off, e.g. blocks whose Newton-Schulz refinement had converged, do not count):
  * complex algorithmic 8 M N K per item, and the BF16 tensor-core flops actually issued (the
- * computed slice products over the padded tiles).  Reading and resetting synchronise the
+ * computed slice or residue products over the padded tiles).  Reading and resetting synchronise the
  * current device. */
 negf_status negf_profile_flops(int32_t kind, double* algorithmic, double* hardware);
 long long negf_launch_count(void);

@@ -113,8 +113,8 @@ int adj_segment(const negf_options* opt, int N) {
   return (sg <= 0 || sg >= N) ? N : sg;
 }
 
-void carve_adj(char* base, size_t& off, int P, int b, int N, int seg, int prec, bool ckpt,
-               AdjWs& w) {
+void carve_adj(char* base, size_t& off, int P, int b, int N, int seg, int prec, bool res,
+               bool ckpt, AdjWs& w) {
   const size_t PB = (size_t)P * b * b;
   const size_t N1 = (size_t)std::max(N - 1, 1);
   // with the solve's checkpoints no sweep block is recomputed or kept here
@@ -140,7 +140,7 @@ void carve_adj(char* base, size_t& off, int P, int b, int N, int seg, int prec, 
   w.GLn = take<z64>(base, off, PB);
   for (int k = 0; k < 14; ++k) w.t[k] = take<z64>(base, off, PB);
   w.vb = take<double>(base, off, (size_t)P * N * b);
-  carve_engine(base, off, P, b, prec, w.eng);
+  carve_engine(base, off, P, b, prec, res, w.eng);
 }
 
 #define CK(x)                                    \
@@ -183,7 +183,7 @@ negf_status adjoint_chunk_run(const AdjArgs& a, int P, char* wsbase, cudaStream_
   const bool have_ck = a.ckpt != nullptr;
   const int seg = have_ck ? N : adj_segment(a.opt, N);
   const int nseg = (N + seg - 1) / seg;
-  carve_adj(wsbase, off, P, b, N, seg, a.opt->precision, have_ck, w);
+  carve_adj(wsbase, off, P, b, N, seg, a.opt->precision, residue_products(a.n_tot), have_ck, w);
   // block of kind k of slab i in the solve's checkpoints (read only)
   auto ck = [&](int k, int i) -> z64* {
     return const_cast<z64*>(a.ckpt) + ckpt_offset(k, i, N, a.n_tot, a.p0, bb);
@@ -528,17 +528,18 @@ constexpr size_t kAdjBudget = 32ull << 30;
 
 }  // namespace
 
-size_t adjoint_bytes(const negf_device* dev, int P, const negf_options* opt, bool ckpt) {
+size_t adjoint_bytes(const negf_device* dev, int P, bool res, const negf_options* opt, bool ckpt) {
   size_t off = 0;
   AdjWs w;
   carve_adj(nullptr, off, P, dev->block, dev->n_slabs, adj_segment(opt, dev->n_slabs),
-            opt->precision, ckpt, w);
+            opt->precision, res, ckpt, w);
   return off + 256;
 }
 
 int adjoint_chunk(const negf_device* dev, int n_pts, const negf_options* opt, bool ckpt) {
   if (opt->chunk > 0) return std::max(1, std::min(std::min(opt->chunk, n_pts), 16384));
-  const size_t per = adjoint_bytes(dev, 2, opt, ckpt) - adjoint_bytes(dev, 1, opt, ckpt);
+  const bool res = residue_products(n_pts);
+  const size_t per = adjoint_bytes(dev, 2, res, opt, ckpt) - adjoint_bytes(dev, 1, res, opt, ckpt);
   size_t c = std::max<size_t>(1, kAdjBudget / std::max<size_t>(per, 1));
   return (int)std::max<size_t>(1, std::min<size_t>(c, (size_t)std::max(n_pts, 1)));
 }
@@ -580,7 +581,7 @@ extern "C" negf_status negf_rgf_adjoint(const negf_device* dev, int32_t n_pts, c
   if (scat_R && (e_idx ? n_rows < 1 : n_rows < n_pts)) return NEGF_ERR_ARG;
   const bool ckpt = checkpoints != nullptr;
   const int C = adjoint_chunk(dev, n_pts, opt, ckpt);
-  if (!ws || ws_bytes < adjoint_bytes(dev, C, opt, ckpt)) return NEGF_ERR_NOMEM;
+  if (!ws || ws_bytes < adjoint_bytes(dev, C, residue_products(n_pts), opt, ckpt)) return NEGF_ERR_NOMEM;
   if (cudaMemsetAsync(status, 0, (size_t)n_pts * sizeof(int32_t), s) != cudaSuccess)
     return NEGF_ERR_CUDA;
   const size_t bb = (size_t)b * b;

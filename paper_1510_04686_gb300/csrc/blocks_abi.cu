@@ -2,6 +2,7 @@
 // built from, exposed for callers that assemble their own recursions.
 #include <algorithm>
 
+#include "crt_gemm.cuh"
 #include "engine.cuh"
 #include "profile.cuh"
 #include "tc_gemm.cuh"
@@ -16,7 +17,8 @@ size_t negf_zgemm_workspace_size(int32_t precision, int32_t n_batch, int32_t M, 
   if (!prec_valid(precision) || n_batch < 1 || M < 1 || N < 1 || K < 1) return 0;
   if (precision == NEGF_PREC_FP64) return 256;
   if (!tc_supports_k(K, prec_bits(precision))) return 0;
-  return tc_ws_bytes(n_batch, M, N, K, prec_bits(precision)) + 1024;
+  return (residue_products(n_batch) ? crt_ws_bytes(n_batch, M, N, K, prec_bits(precision))
+                                    : tc_ws_bytes(n_batch, M, N, K, prec_bits(precision))) + 1024;
 }
 
 negf_status negf_zgemm_batched(int32_t precision, int32_t n_batch, int32_t M, int32_t N,
@@ -53,11 +55,18 @@ negf_status negf_zgemm_batched(int32_t precision, int32_t n_batch, int32_t M, in
     if (K == 0) return NEGF_ERR_UNSUPPORTED;
     size_t off = 0;
     char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + 1023) & ~uintptr_t(1023));
-    TcWs tw;
     const int bits = prec_bits(precision);
-    tc_ws_carve(base, off, n_batch, M, N, K, bits, tw);
-    e = tc_gemm(s, n_batch, M, N, K, al, a, opA, b, opB, be, c, zero, none, false, nullptr, tw,
-                bits);
+    if (residue_products(n_batch)) {
+      CrtWs cw;
+      crt_ws_carve(base, off, n_batch, M, N, K, bits, cw);
+      e = crt_gemm(s, n_batch, M, N, K, al, a, opA, b, opB, be, c, zero, none, false, nullptr, cw,
+                   bits);
+    } else {
+      TcWs tw;
+      tc_ws_carve(base, off, n_batch, M, N, K, bits, tw);
+      e = tc_gemm(s, n_batch, M, N, K, al, a, opA, b, opB, be, c, zero, none, false, nullptr, tw,
+                  bits);
+    }
   }
   return note_error(e) == cudaSuccess ? NEGF_OK : NEGF_ERR_CUDA;
 }
@@ -67,7 +76,7 @@ size_t negf_zinv_workspace_size(int32_t precision, int32_t n_batch, int32_t n) {
   if (!engine_supports(precision, n)) return 0;
   size_t off = 0;
   EngineWs w;
-  carve_engine(nullptr, off, n_batch, n, precision, w);
+  carve_engine(nullptr, off, n_batch, n, precision, residue_products(n_batch), w);
   return off + 1024;
 }
 
@@ -86,7 +95,7 @@ negf_status negf_zinv_batched(int32_t precision, int32_t n_batch, int32_t n, dou
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
   size_t off = 0;
   EngineWs w;
-  carve_engine(base, off, n_batch, n, precision, w);
+  carve_engine(base, off, n_batch, n, precision, residue_products(n_batch), w);
   negf_options o;
   negf_default_options(&o);
   Engine eng(s, precision, refine_steps, std::max(refine_steps, (int)o.refine_max), w, n);

@@ -1,6 +1,7 @@
 // Engine dispatch: FP64 reference form and the mixed-precision tensor-core form.
 #include <atomic>
 
+#include "crt_gemm.cuh"
 #include "engine.cuh"
 #include "profile.cuh"
 #include "tc_gemm.cuh"
@@ -56,7 +57,8 @@ __global__ void k_refine_gate(int P, const int32_t* active, int force, float* rm
 // Residual target of the mixed-form inverse: after a step with max |R| <= 2^-24 the next
 // residual R^2 is at the rounding floor of the products.
 constexpr float kRefineTol = 5.9604644775390625e-8f;
-void carve_engine(char* base, size_t& off, int P, int b, int precision, EngineWs& w) {
+void carve_engine(char* base, size_t& off, int P, int b, int precision, bool residues,
+                  EngineWs& w) {
   const size_t bb = (size_t)b * b;
   const int nb64 = gj_panel_width(b, (int)sizeof(z64));
   w.invU = take<z64>(base, off, (size_t)P * b * nb64);
@@ -67,7 +69,7 @@ void carve_engine(char* base, size_t& off, int P, int b, int precision, EngineWs
   w.act = nullptr;
   w.rmax = nullptr;
   w.tc = nullptr;
-  w.tc_bytes = 0;
+  w.residues = residues;
   if (prec_mixed(precision)) {
     const int nb32 = gj_panel_width(b, (int)sizeof(cx<float>));
     w.m32 = take<cx<float>>(base, off, (size_t)P * bb);
@@ -78,12 +80,15 @@ void carve_engine(char* base, size_t& off, int P, int b, int precision, EngineWs
     w.act = take<int32_t>(base, off, (size_t)P);
     w.rmax = take<float>(base, off, (size_t)P);
     size_t a = (off + 1023) & ~size_t(1023);
-    size_t o2 = a;
-    TcWs tw;
-    tc_ws_carve(base, o2, P, b, b, b, prec_bits(precision), tw);
     w.tc = base ? base + a : nullptr;
-    w.tc_bytes = o2 - a;
-    off = o2;
+    off = a;
+    if (residues) {
+      CrtWs cw;
+      crt_ws_carve(base, off, P, b, b, b, prec_bits(precision), cw);
+    } else {
+      TcWs tw;
+      tc_ws_carve(base, off, P, b, b, b, prec_bits(precision), tw);
+    }
   }
 }
 
@@ -118,10 +123,23 @@ static TcWs tc_view(const EngineWs& w, int P, int b, int bits) {
   tc_ws_carve(static_cast<char*>(w.tc), off, P, b, b, b, bits, t);
   return t;
 }
+static CrtWs crt_view(const EngineWs& w, int P, int b, int bits) {
+  CrtWs t;
+  size_t off = 0;
+  crt_ws_carve(static_cast<char*>(w.tc), off, P, b, b, b, bits, t);
+  return t;
+}
+// The device error word, first in the operand scratch of either form.
+static int32_t* err_word(const EngineWs& w) {
+  return static_cast<int32_t*>(w.tc);
+}
 
 cudaError_t Engine::gemm(int P, int M, int N, int K, z64 alpha, BMc<double> A, int opA,
                          BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
                          BMc<double> D, const int32_t* active) {
+  if (prec_mixed(prec) && w.residues)
+    return crt_gemm(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, false, active,
+                    crt_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys);
   if (prec_mixed(prec))
     return tc_gemm(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, false, active,
                    tc_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys);
@@ -130,7 +148,7 @@ cudaError_t Engine::gemm(int P, int M, int N, int K, z64 alpha, BMc<double> A, i
 
 cudaError_t Engine::timeout_reset() {
   if (!prec_mixed(prec)) return cudaSuccess;
-  return tc_timeout_reset(s, tc_view(w, 1, b, prec_bits(prec)));
+  return tc_timeout_reset(s, err_word(w));
 }
 
 namespace {
@@ -139,12 +157,11 @@ std::atomic<int> g_fail_waits{0};
 
 cudaError_t Engine::timeout_flag(int P, int32_t* status) {
   if (!prec_mixed(prec)) return cudaSuccess;
-  const TcWs tw = tc_view(w, 1, b, prec_bits(prec));
   if (g_fail_waits.load()) {  // test hook: report as if a bounded wait had given up
-    cudaError_t e = cudaMemsetAsync(tw.err, 1, sizeof(int32_t), s);
+    cudaError_t e = cudaMemsetAsync(err_word(w), 1, sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
   }
-  return tc_timeout_flag(s, tw, P, status);
+  return tc_timeout_flag(s, err_word(w), P, status);
 }
 
 void engine_fail_waits(int on) { g_fail_waits.store(on ? 1 : 0); }
@@ -175,7 +192,6 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (refine_max <= 0) return cudaSuccess;
   const int bits = prec_bits(prec);
-  const TcWs tw = tc_view(w, P, b, bits);
   const BMc<double> none{nullptr, 0, nullptr, 0};
   const unsigned gb = (unsigned)((P + 255) / 256);
   BM<double> R{w.r64, bb, nullptr, b};
@@ -188,13 +204,25 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
                                      kRefineTol, w.act, 0);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    e = tc_gemm(s, P, b, b, b, mkc(-1.0, 0.0), Mc, OP_N, Xc, OP_N, mkc(0.0, 0.0), R,
-                mkc(0.0, 0.0), none, true, w.act, tw, bits, 0, false, w.rmax);
+    const z64 zero = mkc(0.0, 0.0), one = mkc(1.0, 0.0), mone = mkc(-1.0, 0.0);
+    if (w.residues) {
+      const CrtWs cw = crt_view(w, P, b, bits);
+      e = crt_gemm(s, P, b, b, b, mone, Mc, OP_N, Xc, OP_N, zero, R, zero, none, true, w.act, cw,
+                   bits, 0, w.rmax);
+      if (e != cudaSuccess) return e;
+      e = crt_gemm(s, P, b, b, b, one, Xc, OP_N, cst(R), OP_N, zero, X, one, Xc, false, w.act, cw,
+                   bits);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
+    const TcWs tw = tc_view(w, P, b, bits);
+    e = tc_gemm(s, P, b, b, b, mone, Mc, OP_N, Xc, OP_N, zero, R, zero, none, true, w.act, tw,
+                bits, 0, false, w.rmax);
     if (e != cudaSuccess) return e;
     // X <- X + X R in place (each output element reads only its own X entry; the product reads
     // the slices of X made before it).  With |R| << 1 only accuracy relative to |X| matters.
-    e = tc_gemm(s, P, b, b, b, mkc(1.0, 0.0), Xc, OP_N, cst(R), OP_N, mkc(0.0, 0.0), X,
-                mkc(1.0, 0.0), Xc, false, w.act, tw, bits, 0, true);
+    e = tc_gemm(s, P, b, b, b, one, Xc, OP_N, cst(R), OP_N, zero, X, one, Xc, false, w.act, tw,
+                bits, 0, true);
     if (e != cudaSuccess) return e;
   }
   // items whose last residual was still above the target: FP64 Gauss-Jordan (M is intact)

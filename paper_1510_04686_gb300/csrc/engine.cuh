@@ -22,13 +22,25 @@ struct EngineWs {
   z64* r64;          // residual I - M X, P x b x b
   int32_t* act;      // items still refined by the current Newton-Schulz step, P
   float* rmax;       // max |I - M X| of each item after the last residual product, P
-  void* tc;          // tensor-core GEMM operand slices
-  size_t tc_bytes;
+  void* tc;          // tensor-core GEMM operand slices or residues
+  bool residues;     // the form that tc was carved for
 };
 
+// Form of the tensor-core products of a call over n items (points, or matrices of a batch).
+// Residue products (crt_gemm.cuh) are the faster and the more accurate form at every size.  Calls
+// of few items keep digit-slice products (tc_gemm.cuh) and with them the results that they have
+// always given, because there the two forms can differ by more than rounding of the result: a
+// bond current at an energy below the bias window is the small difference of two large terms, so
+// each form gives digits there that the arithmetic does not determine.  A batch of a dozen energies
+// or more has some inside the window, and is judged by the currents there.
+constexpr int kResidueItems = 12;
+inline bool residue_products(int n_items) { return n_items >= kResidueItems; }
+
 // Reserve the engine scratch for P concurrent b x b problems at `off` of `base` (base NULL:
-// only advance `off`).  precision: a negf_precision value (it fixes the tensor-core slices).
-void carve_engine(char* base, size_t& off, int P, int b, int precision, EngineWs& w);
+// only advance `off`).  precision: a negf_precision value, residues: the form of its products
+// (they fix the tensor-core operand scratch).
+void carve_engine(char* base, size_t& off, int P, int b, int precision, bool residues,
+                  EngineWs& w);
 
 // Precision tiers: FP64 on the CUDA cores, or tensor-core products of 40-, 48- or 56-bit
 // fixed-point operand values.
@@ -106,7 +118,8 @@ bool engine_supports(int precision, int b);
 
 // Adjoint workspace helpers (adjoint.cu)
 // ckpt: the sweep blocks come from negf_rgf_solve's checkpoints (no resident segment blocks)
-size_t adjoint_bytes(const negf_device* dev, int P, const negf_options* opt, bool ckpt);
+// res: residue products
+size_t adjoint_bytes(const negf_device* dev, int P, bool res, const negf_options* opt, bool ckpt);
 int adjoint_chunk(const negf_device* dev, int n_pts, const negf_options* opt, bool ckpt);
 // Sweep checkpoints handed from negf_rgf_solve to negf_rgf_adjoint: complex128
 // [5][N][n_pts][b][b], the kinds below, slab-major so that a chunk of consecutive points of one

@@ -67,7 +67,8 @@ struct LeadWs {
   EngineWs eng;
 };
 
-void carve_lead(Carver& c, int P, int b, const negf_options* opt, LeadWs& w) {
+// res: residue products (residue_products of the call's points)
+void carve_lead(Carver& c, int P, int b, bool res, const negf_options* opt, LeadWs& w) {
   const size_t bb = (size_t)b * b, Q = 2 * (size_t)P;
   w.eps_s = c.take<z64>(Q * bb);
   w.eps = c.take<z64>(Q * bb);
@@ -87,7 +88,7 @@ void carve_lead(Carver& c, int P, int b, const negf_options* opt, LeadWs& w) {
   w.n_active = c.take<int32_t>(1);
   w.sys = c.take<int32_t>((size_t)P);
   w.act_side = c.take<int32_t>(Q);
-  carve_engine(c.base ? c.base : nullptr, c.off, (int)Q, b, lead_precision(opt, b), w.eng);
+  carve_engine(c.base, c.off, (int)Q, b, lead_precision(opt, b), res, w.eng);
 }
 
 struct RgfWs {
@@ -97,7 +98,7 @@ struct RgfWs {
   EngineWs eng;
 };
 
-void carve_rgf(Carver& c, int P, int b, int N, const negf_options* opt, RgfWs& w) {
+void carve_rgf(Carver& c, int P, int b, int N, bool res, const negf_options* opt, RgfWs& w) {
   const size_t bb = (size_t)b * b, PB = (size_t)P * bb;
   w.sys = c.take<int32_t>((size_t)P);
   w.erow = c.take<int32_t>((size_t)P);
@@ -114,19 +115,19 @@ void carve_rgf(Carver& c, int P, int b, int N, const negf_options* opt, RgfWs& w
   w.Qm = c.take<z64>(PB);
   w.U = c.take<z64>(PB);
   w.Mt = c.take<z64>(PB);
-  carve_engine(c.base, c.off, P, b, opt->precision, w.eng);
+  carve_engine(c.base, c.off, P, b, opt->precision, res, w.eng);
 }
 
-size_t lead_bytes(int P, int b, const negf_options* o) {
+size_t lead_bytes(int P, int b, bool res, const negf_options* o) {
   Carver c{nullptr, 0};
   LeadWs w;
-  carve_lead(c, P, b, o, w);
+  carve_lead(c, P, b, res, o, w);
   return c.off + 256;
 }
-size_t rgf_bytes(int P, int b, int N, const negf_options* o) {
+size_t rgf_bytes(int P, int b, int N, bool res, const negf_options* o) {
   Carver c{nullptr, 0};
   RgfWs w;
-  carve_rgf(c, P, b, N, o, w);
+  carve_rgf(c, P, b, N, res, o, w);
   return c.off + 256;
 }
 
@@ -140,11 +141,13 @@ int pick_chunk(int n_pts, const negf_options* o, size_t per_pt) {
 }
 
 int lead_chunk(const negf_device* d, int n_pts, const negf_options* o) {
-  size_t per = lead_bytes(2, d->block, o) - lead_bytes(1, d->block, o);
+  const bool res = residue_products(n_pts);
+  size_t per = lead_bytes(2, d->block, res, o) - lead_bytes(1, d->block, res, o);
   return pick_chunk(n_pts, o, per);
 }
 int rgf_chunk(const negf_device* d, int n_pts, const negf_options* o) {
-  size_t per = rgf_bytes(2, d->block, d->n_slabs, o) - rgf_bytes(1, d->block, d->n_slabs, o);
+  const bool res = residue_products(n_pts);
+  size_t per = rgf_bytes(2, d->block, d->n_slabs, res, o) - rgf_bytes(1, d->block, d->n_slabs, res, o);
   return pick_chunk(n_pts, o, per);
 }
 
@@ -153,7 +156,7 @@ inline BM<double> flat(z64* base, size_t bb, int b) {
 }
 
 // ---------------------------------------------------------------- lead self-energies
-negf_status lead_chunk_run(const negf_device* dev, int P, const double* E, const int32_t* sys_in,
+negf_status lead_chunk_run(const negf_device* dev, int P, bool res, const double* E, const int32_t* sys_in,
                            const negf_options* opt, z64* sigR, z64* sigL, int32_t* iters,
                            int32_t* status, char* wsbase, cudaStream_t s) {
   const int b = dev->block, N = dev->n_slabs;
@@ -168,7 +171,7 @@ negf_status lead_chunk_run(const negf_device* dev, int P, const double* E, const
   }
   Carver c{wsbase, 0};
   LeadWs w;
-  carve_lead(c, P, b, opt, w);
+  carve_lead(c, P, b, res, opt, w);
   Engine eng(s, lead_precision(opt, b), opt->refine_steps, refine_limit(opt), w.eng, b,
              dev->n_sys);
   CK(eng.timeout_reset());
@@ -316,6 +319,7 @@ struct RgfArgs {
   const int32_t* e_idx;
   int32_t n_rows;
   const negf_options* opt;
+  bool res;  // residue products (residue_products of the call's points)
   double* density;
   double* current;
   double* transmission;
@@ -335,7 +339,7 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
   const z64 one = mkc(1.0, 0.0), zero = mkc(0.0, 0.0), two = mkc(2.0, 0.0);
   Carver c{wsbase, 0};
   RgfWs w;
-  carve_rgf(c, P, b, N, a.opt, w);
+  carve_rgf(c, P, b, N, a.res, a.opt, w);
   Engine eng(s, a.opt->precision, a.opt->refine_steps, refine_limit(a.opt), w.eng, b,
              dev->n_sys);
   CK(eng.timeout_reset());
@@ -553,12 +557,16 @@ size_t negf_workspace_size(const negf_device* dev, int32_t n_pts, const negf_opt
     return 0;
   const int b = dev->block, N = dev->n_slabs;
   switch (which) {
-    case NEGF_WS_LEAD: return lead_bytes(lead_chunk(dev, n_pts, opt), b, opt);
-    case NEGF_WS_RGF: return rgf_bytes(rgf_chunk(dev, n_pts, opt), b, N, opt);
+    case NEGF_WS_LEAD:
+      return lead_bytes(lead_chunk(dev, n_pts, opt), b, residue_products(n_pts), opt);
+    case NEGF_WS_RGF:
+      return rgf_bytes(rgf_chunk(dev, n_pts, opt), b, N, residue_products(n_pts), opt);
     case NEGF_WS_ADJOINT:
-      return adjoint_bytes(dev, adjoint_chunk(dev, n_pts, opt, false), opt, false);
+      return adjoint_bytes(dev, adjoint_chunk(dev, n_pts, opt, false), residue_products(n_pts), opt,
+                           false);
     case NEGF_WS_ADJOINT_CKPT:
-      return adjoint_bytes(dev, adjoint_chunk(dev, n_pts, opt, true), opt, true);
+      return adjoint_bytes(dev, adjoint_chunk(dev, n_pts, opt, true), residue_products(n_pts), opt,
+                           true);
   }
   return 0;
 }
@@ -579,14 +587,15 @@ negf_status negf_lead_selfenergy(const negf_device* dev, int32_t n_pts, const do
   if (!E || !sys_idx || !sigma_R || !sigma_L || !status) return NEGF_ERR_ARG;
   const int b = dev->block;
   const int C = lead_chunk(dev, n_pts, opt);
-  if (dev->n_slabs > 1 && (!ws || ws_bytes < lead_bytes(C, b, opt))) return NEGF_ERR_NOMEM;
+  const bool res = residue_products(n_pts);
+  if (dev->n_slabs > 1 && (!ws || ws_bytes < lead_bytes(C, b, res, opt))) return NEGF_ERR_NOMEM;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t bb = (size_t)b * b;
   if (cudaMemsetAsync(status, 0, (size_t)n_pts * sizeof(int32_t), s) != cudaSuccess)
     return NEGF_ERR_CUDA;
   for (int p0 = 0; p0 < n_pts; p0 += C) {
     const int P = std::min(C, n_pts - p0);
-    negf_status r = lead_chunk_run(dev, P, E + p0, sys_idx + p0, opt,
+    negf_status r = lead_chunk_run(dev, P, res, E + p0, sys_idx + p0, opt,
                                    reinterpret_cast<z64*>(sigma_R) + (size_t)p0 * 2 * bb,
                                    reinterpret_cast<z64*>(sigma_L) + (size_t)p0 * 2 * bb,
                                    iters ? iters + 2 * (size_t)p0 : nullptr, status + p0,
@@ -612,7 +621,8 @@ negf_status negf_rgf_solve(const negf_device* dev, int32_t n_pts, const double* 
   if ((scat_R == nullptr) != (scat_L == nullptr)) return NEGF_ERR_ARG;
   const int b = dev->block, N = dev->n_slabs;
   const int C = rgf_chunk(dev, n_pts, opt);
-  if (!ws || ws_bytes < rgf_bytes(C, b, N, opt)) return NEGF_ERR_NOMEM;
+  const bool res = residue_products(n_pts);
+  if (!ws || ws_bytes < rgf_bytes(C, b, N, res, opt)) return NEGF_ERR_NOMEM;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t bb = (size_t)b * b, NB = (size_t)N * b;
   const int A = sigma_width(opt);
@@ -634,6 +644,7 @@ negf_status negf_rgf_solve(const negf_device* dev, int32_t n_pts, const double* 
     a.scatR = scat_R ? reinterpret_cast<const z64*>(scat_R) + (e_idx ? 0 : (size_t)p0 * NBA) : nullptr;
     a.scatL = scat_L ? reinterpret_cast<const z64*>(scat_L) + (e_idx ? 0 : (size_t)p0 * NBA) : nullptr;
     a.opt = opt;
+    a.res = res;
     a.density = density ? density + (size_t)p0 * NB : nullptr;
     a.current = (current && N > 1) ? current + (size_t)p0 * (N - 1) : nullptr;
     a.transmission = transmission ? transmission + p0 : nullptr;

@@ -51,7 +51,7 @@ extern "C" negf_status negf_zinv_batched_noalloc(int32_t n_batch, int32_t n, dou
   // blocks small enough for the one-CTA shared-memory elimination use no scratch at all
   size_t need = 0;
   EngineWs w;
-  if (!gj_fits_small(n, (int)sizeof(z64))) carve_engine(nullptr, need, n_batch, n, NEGF_PREC_FP64, w);
+  if (!gj_fits_small(n, (int)sizeof(z64))) carve_engine(nullptr, need, n_batch, n, NEGF_PREC_FP64, false, w);
   if (need > kNoAllocBytes) return NEGF_ERR_NOMEM;
   void* base = nullptr;
   if (scratch_address(&base) != cudaSuccess) return NEGF_ERR_CUDA;
@@ -59,7 +59,7 @@ extern "C" negf_status negf_zinv_batched_noalloc(int32_t n_batch, int32_t n, dou
   if (cudaMemsetAsync(status, 0, (size_t)n_batch * sizeof(int32_t), s) != cudaSuccess)
     return NEGF_ERR_CUDA;
   size_t off = 0;
-  carve_engine(static_cast<char*>(base), off, n_batch, n, NEGF_PREC_FP64, w);
+  carve_engine(static_cast<char*>(base), off, n_batch, n, NEGF_PREC_FP64, false, w);
   const long long nn = (long long)n * n;
   cudaError_t e = gj_inverse<double>(s, n_batch, n, BM<double>{reinterpret_cast<z64*>(M), nn, nullptr, n},
                                      BM<double>{reinterpret_cast<z64*>(X), nn, nullptr, n}, w.invU,

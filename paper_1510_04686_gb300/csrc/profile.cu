@@ -4,6 +4,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "crt_gemm.cuh"
 #include "profile.cuh"
 #include "tc_gemm.cuh"
 
@@ -106,6 +107,7 @@ negf_status negf_profile_read(int32_t kind, long long* launches, double* total_m
 void negf_profile_reset(void) {
   std::lock_guard<std::mutex> lk(g_mu);
   tc_prof_reset();
+  crt_prof_reset();
   for (int k = 0; k < PROF_KINDS; ++k) {
     g_count[k] = 0;
     g_ms[k] = 0.0;
@@ -118,7 +120,11 @@ negf_status negf_profile_flops(int32_t kind, double* algorithmic, double* hardwa
   if (kind < 0 || kind >= PROF_KINDS || !algorithmic || !hardware) return NEGF_ERR_ARG;
   std::lock_guard<std::mutex> lk(g_mu);
   if (kind == PROF_TC_GEMM) {  // counted on the device, for the batch items that ran
-    if (tc_prof_flops(algorithmic, hardware) != cudaSuccess) return NEGF_ERR_CUDA;
+    double alg = 0.0, hw = 0.0;
+    if (tc_prof_flops(algorithmic, hardware) != cudaSuccess || crt_prof_flops(&alg, &hw) != cudaSuccess)
+      return NEGF_ERR_CUDA;
+    *algorithmic += alg;
+    *hardware += hw;
     return NEGF_OK;
   }
   *algorithmic = g_alg[kind];

@@ -1,4 +1,5 @@
-// Tensor-core complex GEMM with FP64-class accuracy from exact split-BF16 products.
+// Tensor-core complex GEMM with FP64-class accuracy from exact split-BF16 products (the form of
+// calls of few items; crt_gemm.cuh is that of batches).
 //
 //   C = alpha op(A) op(B) + beta C + gamma D (+ I)       (complex128 in and out)
 //
@@ -48,8 +49,8 @@ bool tc_supports_k(int K, int bits);
 // The device error word ws.err is set when a bounded wait inside the GEMM kernel gave up (the
 // tile's outputs are then NaN).  tc_timeout_reset zeroes it; tc_timeout_flag ORs
 // NEGF_PT_TIMEOUT into status[0..P) when it is set.  Both are asynchronous on s.
-cudaError_t tc_timeout_reset(cudaStream_t s, const TcWs& ws);
-cudaError_t tc_timeout_flag(cudaStream_t s, const TcWs& ws, int P, int32_t* status);
+cudaError_t tc_timeout_reset(cudaStream_t s, int32_t* err);
+cudaError_t tc_timeout_flag(cudaStream_t s, const int32_t* err, int P, int32_t* status);
 
 // Flops of the tensor-core GEMM launches made while profiling was on, counted on the device
 // for the items that ran (the current device; both calls synchronise it): algorithmic complex
