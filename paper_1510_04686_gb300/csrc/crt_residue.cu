@@ -170,82 +170,6 @@ __device__ __forceinline__ void write_planes(const ResidueConst& rc, const Coef&
 // neighbouring values of a residue plane and stores them as 16 bytes, 128 contiguous bytes per
 // plane and warp.  Bound by instruction issue (450 per value and 12 moduli; 2.85 us per 400 x 400
 // operand, 3.6 TB/s of reads and writes).
-constexpr int kThreads = 256, kWarps = kThreads / 32;
-// a pad of one entry after every eight keeps the digit loads free of bank conflicts
-__host__ __device__ constexpr int padded(int k) { return k + (k >> 3); }
-// The constants in shared memory (a lane-dependent index into the kernel's parameters is served
-// one lane at a time, once per CTA instead of once per warp); padded rows.
-typedef uint32_t Coef[2 * kMaxMod][kDigits + 1];
-__device__ __forceinline__ void load_coef(const ResidueConst& rc, Coef& coef) {
-  for (int i = threadIdx.x; i < 2 * kMaxMod * kDigits; i += blockDim.x)
-    coef[i / kDigits][i % kDigits] = reinterpret_cast<const uint32_t*>(&rc.coef[0][0])[i];
-}
-
-// The residue planes of lines l0 .. l0 + LINES - 1, elements k0 .. k0 + len - 1 (multiples of 8),
-// from their biased integers in shared memory.
-template <int LINES, int NB>
-__device__ __forceinline__ void write_planes(const ResidueConst& rc, const Coef& coef, int n,
-                                             const ulonglong2* ints,
-                                             int lds, int l0, int n_lines, int k0, int len, int L,
-                                             __nv_bfloat16* base) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // lane (g, t) holds columns 2 t, 2 t + 1 of a digit matrix and, of every eight results, the
-  // pair (u, v) of modulus 4 b + t
-  const int g = lane >> 2, t = lane & 3;
-  const uint32_t sel = (uint32_t)(2 * t) | (uint32_t)(2 * t + 1) << 8;
-  uint32_t b0[NB], b1[NB];
-  f2 invp[NB], negp[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const int col = 8 * b + g, l = min(4 * b + t, n - 1);
-    b0[b] = coef[col][t];
-    b1[b] = coef[col][t + 4];
-    invp[b] = pack2(rc.invp[l], rc.invp[l]);
-    negp[b] = pack2(rc.negp[l], rc.negp[l]);
-  }
-  const long long plane = (long long)n_lines * L;  // one residue plane of an item
-  const int blocks = (len + 63) / 64;
-  for (int job = w; job < LINES * blocks; job += kWarps) {
-    const int line = job / blocks, kb = (job - line * blocks) * 64 + 8 * g;
-    if (l0 + line >= n_lines) break;
-    const bool in = kb < len;
-    const ulonglong2* row = ints + line * lds + padded(in ? kb : 0);
-    uint32_t u[NB][4], v[NB][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const ulonglong2 e0 = row[2 * i], e1 = row[2 * i + 1];
-      const uint32_t a[4] = {digit_pair(e0.x, sel), digit_pair(e1.x, sel),
-                             digit_pair(e0.y, sel), digit_pair(e1.y, sel)};
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        float d[4];
-        mma_16x8x16(d, a, b0[b], b1[b]);
-        u[b][i] = residue_bf16(d[0], d[2], invp[b], negp[b]);
-        v[b][i] = residue_bf16(d[1], d[3], invp[b], negp[b]);
-      }
-    }
-    if (!in) continue;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int l = 4 * b + t;
-      if (l < n) {
-        __nv_bfloat16* o = base + 2 * l * plane + (long long)(l0 + line) * L + k0 + kb;
-        *reinterpret_cast<uint4*>(o) = make_uint4(u[b][0], u[b][1], u[b][2], u[b][3]);
-        *reinterpret_cast<uint4*>(o + plane) = make_uint4(v[b][0], v[b][1], v[b][2], v[b][3]);
-      }
-    }
-  }
-}
-
-// Residues of LINES lines per CTA.  The strip (LINES lines of K complex values) is read once,
-// coalesced along the operand's memory layout, with the norms taken on the way; its values become
-// biased 64-bit integers in shared memory.  A warp then takes 64 values of a line at a time: four
-// 16 x 16 digit matrices (rows: values, columns: the digits of Re and Im) times the 16 x 2 n
-// constants, whose results are reduced modulo p in registers; a lane ends up with eight
-// neighbouring values of a residue plane and stores them as 16 bytes, 128 contiguous bytes per
-// plane and warp.  Bound by the residues written (48 bytes per value at n = 12) once the digit
-// sums run on the tensor core: as FP32 multiply-adds per value and modulus they took twice the
-// time of the stores.
 template <int LINES, int NB>
 __global__ void __launch_bounds__(kThreads)
     k_residue_strip(const __grid_constant__ ResidueConst rc, int n, int alpha, double sigma,
