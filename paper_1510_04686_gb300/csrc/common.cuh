@@ -109,12 +109,16 @@ cudaError_t gemm_simt(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc
                       const int32_t* active);
 
 // X[p] = M[p]^-1 by Gauss-Jordan elimination with partial pivoting (largest |m|, lowest row
-// on ties, pivots compared in FP64).  M is destroyed.  A zero pivot sets NEGF_PT_SINGULAR in
-// status[p] and is replaced by a tiny number so the sweep continues.
-// Scratch: U (P x n x nb), T (P x nb x n), piv (P x n) from gj_scratch_elems().
-template <typename R>
-cudaError_t gj_inverse(cudaStream_t s, int P, int n, BM<R> M, BM<R> X, cx<R>* U, cx<R>* T,
-                       int32_t* piv, int32_t* status, const int32_t* active);
+// on ties, pivots compared in FP64).  A zero pivot sets NEGF_PT_SINGULAR in status[p] and is
+// replaced by a tiny number so the sweep continues.  Scratch: piv (P x n).
+// FP64: M is destroyed; scratch U (P x n x nb), T (P x nb x n), nb = gj_panel_width(n, 16).
+// FP32: elimination in FP32 (m32 and x32: P x n x n, U: P x n x nb, nb = gj_panel_width(n, 8), map:
+// P x n), M is kept; M and X are contiguous n x n blocks.
+cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, z64* U, z64* T,
+                         int32_t* piv, int32_t* status, const int32_t* active);
+cudaError_t gj_inverse32(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, cx<float>* m32,
+                         cx<float>* x32, cx<float>* U, int32_t* piv, int32_t* map, int32_t* status,
+                         const int32_t* active);
 int gj_panel_width(int n, int elem_bytes);
 bool gj_fits_small(int n, int elem_bytes);
 // Whether the batched Gauss-Jordan inverse launches for n x n blocks of elem_bytes complex

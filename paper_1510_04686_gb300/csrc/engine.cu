@@ -16,26 +16,6 @@ T* take(char* base, size_t& off, size_t n) {
   return base ? reinterpret_cast<T*>(base + a) : nullptr;
 }
 
-__global__ void k_to32(long long n, const z64* a, cx<float>* o, const int32_t* active,
-                       long long per) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    if (active && !active[k / per]) continue;
-    o[k] = mkc<float>((float)a[k].re, (float)a[k].im);
-  }
-}
-__global__ void k_to64(long long n, const cx<float>* a, z64* o, const int32_t* active,
-                       long long per) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    if (active && !active[k / per]) continue;
-    o[k] = mkc<double>((double)a[k].re, (double)a[k].im);
-  }
-}
-inline unsigned nblk(long long n) {
-  long long b = (n + 255) / 256;
-  return (unsigned)(b > 152 * 32 ? 152 * 32 : (b < 1 ? 1 : b));
-}
 }  // namespace
 
 __device__ unsigned long long g_fp64_fallbacks;  // items recomputed by the FP64 fallback
@@ -64,7 +44,8 @@ void carve_engine(char* base, size_t& off, int P, int b, int precision, bool res
   w.invU = take<z64>(base, off, (size_t)P * b * nb64);
   w.invT = take<z64>(base, off, (size_t)P * b * nb64);
   w.piv = take<int32_t>(base, off, (size_t)P * b);
-  w.m32 = w.x32 = w.invU32 = w.invT32 = nullptr;
+  w.map = nullptr;
+  w.m32 = w.x32 = w.invU32 = nullptr;
   w.r64 = nullptr;
   w.act = nullptr;
   w.rmax = nullptr;
@@ -72,10 +53,10 @@ void carve_engine(char* base, size_t& off, int P, int b, int precision, bool res
   w.residues = residues;
   if (prec_mixed(precision)) {
     const int nb32 = gj_panel_width(b, (int)sizeof(cx<float>));
+    w.map = take<int32_t>(base, off, (size_t)P * b);
     w.m32 = take<cx<float>>(base, off, (size_t)P * bb);
     w.x32 = take<cx<float>>(base, off, (size_t)P * bb);
     w.invU32 = take<cx<float>>(base, off, (size_t)P * b * nb32);
-    w.invT32 = take<cx<float>>(base, off, (size_t)P * b * nb32);
     w.r64 = take<z64>(base, off, (size_t)P * bb);
     w.act = take<int32_t>(base, off, (size_t)P);
     w.rmax = take<float>(base, off, (size_t)P);
@@ -170,26 +151,18 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
                         const int32_t* active) {
   if (!prec_mixed(prec)) {
     prof_begin(s, PROF_INV);
-    cudaError_t e = gj_inverse<double>(s, P, b, Mm, X, w.invU, w.invT, w.piv, status, active);
+    cudaError_t e = gj_inverse64(s, P, b, Mm, X, w.invU, w.invT, w.piv, status, active);
     prof_end(s, PROF_INV);
     return e;
   }
   // FP32 Gauss-Jordan start X0, then X <- X + X (I - M X) with tensor-core products
-  const long long bb = (long long)b * b, n = (long long)P * bb;
+  const long long bb = (long long)b * b;
   if (Mm.idx || X.idx || Mm.stride != bb || X.stride != bb || Mm.ld != b || X.ld != b)
     return cudaErrorInvalidValue;
-  k_to32<<<nblk(n), 256, 0, s>>>(n, Mm.p, w.m32, active, bb);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  BM<float> m32{w.m32, bb, nullptr, b}, x32{w.x32, bb, nullptr, b};
   prof_begin(s, PROF_INV);
-  e = gj_inverse<float>(s, P, b, m32, x32, w.invU32, w.invT32, w.piv, status, active);
+  cudaError_t e = gj_inverse32(s, P, b, Mm, X, w.m32, w.x32, w.invU32, w.piv, w.map, status, active);
   prof_end(s, PROF_INV);
   if (e != cudaSuccess) return e;
-  k_to64<<<nblk(n), 256, 0, s>>>(n, w.x32, X.p, active, bb);
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (refine_max <= 0) return cudaSuccess;
   const int bits = prec_bits(prec);
   const BMc<double> none{nullptr, 0, nullptr, 0};
@@ -230,7 +203,7 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(s, PROF_INV);
-  e = gj_inverse<double>(s, P, b, Mm, X, w.invU, w.invT, w.piv, status, w.act);
+  e = gj_inverse64(s, P, b, Mm, X, w.invU, w.invT, w.piv, status, w.act);
   prof_end(s, PROF_INV);
   return e;
 }

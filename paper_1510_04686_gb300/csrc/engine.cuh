@@ -14,11 +14,11 @@ struct EngineWs {
   z64* invU;
   z64* invT;
   int32_t* piv;
+  int32_t* map;      // row sources of a panel, then the final column order
   // mixed-precision scratch
   cx<float>* m32;    // FP32 copy of the matrices being inverted, P x b x b
   cx<float>* x32;    // FP32 inverse, P x b x b
   cx<float>* invU32;
-  cx<float>* invT32;
   z64* r64;          // residual I - M X, P x b x b
   int32_t* act;      // items still refined by the current Newton-Schulz step, P
   float* rmax;       // max |I - M X| of each item after the last residual product, P

@@ -9,10 +9,13 @@
 // rank-nb update  A[:, rest] += Panel * A[pivot rows, rest]  (pivot rows zeroed first), which is
 // a batched GEMM.  The column permutation is undone at the end.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
+#include <utility>
 
 #include "common.cuh"
 #include "profile.cuh"
+#include "tc_slice.cuh"
 
 namespace negf {
 
@@ -68,7 +71,7 @@ __device__ __forceinline__ cx<R> pivot_recip(cx<R> a, int32_t* st) {
     int e;
     frexpf(fmaxf(fabsf(a.re), fabsf(a.im)), &e);
     const float ar = ldexpf(a.re, -e), ai = ldexpf(a.im, -e);
-    const float inv = ldexpf(1.0f / (ar * ar + ai * ai), -e);
+    const float inv = ldexpf(1.0f / __fmaf_rn(ar, ar, __fmul_rn(ai, ai)), -e);
     return mkc<float>(ar * inv, -ai * inv);
   }
 }
@@ -330,41 +333,239 @@ __global__ void __launch_bounds__(kThreads) k_gj_panel(int n, int k0, int w, int
   }
 }
 
-// Trailing update of a Gauss-Jordan panel step: C += U T for every item, with U the eliminated
-// panel (n x w, row stride nb), T the pivot rows (w x n) and w <= kMaxPanel (FP32 only: the
-// FP64 blocks would not fit the static shared memory).  An 80 x 80 block of C per CTA (n = 400
-// is 5 x 5 blocks with no padding; 64 x 64 blocks would pad it to 448^2, 25 % more work), each
-// thread 5 x 5 complex accumulators: rows ty + 16 i, columns tx + 16 j.  The whole U and T blocks
-// are staged in shared memory at once (one barrier), and C is read into the accumulators before
-// the multiply-adds so that its latency overlaps the staging.
+// FP32 form of the blocked elimination.  A panel is eliminated in registers, and the trailing
+// update reads the matrix through the panel's row exchanges and writes it to a second buffer, so no
+// pass over the matrix moves rows: src and dst alternate from panel to panel.
+//
+// Panel step: columns [k0, k0 + w) of src (w = W, the panel width, but for a matrix's LAST panel,
+// which may be narrower).  Thread (g, c) keeps rows g, g + kG, ... of column c in registers for all
+// steps; a step exchanges only the pivot column f, the two rows of the exchange and the pivot
+// through shared memory.  Writes the eliminated panel to U and to its columns of dst, the pivot
+// rows, and for every row the source row of its content after the panel's exchanges (cont).
+//
+// Bound by the chain of W steps (pivot search, exchange, update, a barrier between each) on one SM
+// per item: 65 us for 64 items of n = 400, W = 32, where a panel in shared memory on 256 threads
+// that also moved the rows of the whole matrix took 110 us.  512 threads: 1024 spend more on the
+// part of a step that every warp repeats, and a test per slot (instead of filler rows) parted the
+// slots' loads and took 140 us.
+// The multiply-adds of a step are written out, each rounding in its place, so that the result does
+// not depend on how the compiler contracts them.  `other` takes the imaginary part's products in
+// the other order: the elimination has always done so in the rows that its unrolling by four left
+// over, and the results stay the same bit for bit.
+__device__ __forceinline__ cx<float> cmul(cx<float> a, cx<float> b) {
+  return mkc<float>(__fmaf_rn(a.re, b.re, -__fmul_rn(a.im, b.im)),
+                    __fmaf_rn(a.re, b.im, __fmul_rn(a.im, b.re)));
+}
+__device__ __forceinline__ void eliminate(cx<float>& x, cx<float> f, cx<float> p, bool other) {
+  x.re = __fsub_rn(x.re, __fmaf_rn(f.re, p.re, -__fmul_rn(f.im, p.im)));
+  const float t = other ? __fmaf_rn(f.re, p.im, __fmul_rn(f.im, p.re))
+                        : __fmaf_rn(f.im, p.re, __fmul_rn(f.re, p.im));
+  x.im = __fsub_rn(x.im, t);
+}
+// Pivot candidates.  hi + lo of mag2 is brought to h = RN(hi + lo) and the exact rest l, so that the
+// larger sum has the larger h, then the larger l; equal sums go to the lower row.  Keys order like
+// unsigned integers (a candidate's h key is at least 1), so a warp finds its winner with reductions
+// of the integer unit.
+struct Cand {
+  uint32_t h, l;
+  int row;
+};
+__device__ __forceinline__ Cand candidate(cx<float> a, int row) {
+  const Mag<float> m = mag2(a);
+  const float h = __fadd_rn(m.hi, m.lo);
+  const uint32_t l = __float_as_uint(__fsub_rn(m.lo, __fsub_rn(h, m.hi)));
+  return Cand{__float_as_uint(h) + 1u, l & 0x80000000u ? ~l : l | 0x80000000u, row};
+}
+__device__ __forceinline__ bool wins(const Cand& a, const Cand& b) {
+  return a.h > b.h || (a.h == b.h && (a.l > b.l || (a.l == b.l && a.row < b.row)));
+}
+__device__ __forceinline__ Cand warp_winner(Cand c) {
+  const uint32_t full = 0xffffffffu;
+  const uint32_t h = __reduce_max_sync(full, c.h);
+  const uint32_t tied = __ballot_sync(full, c.h == h);
+  int src = __ffs((int)tied) - 1;
+  if (tied & (tied - 1)) {
+    const uint32_t l = __reduce_max_sync(full, c.h == h ? c.l : 0u);
+    const bool in = c.h == h && c.l == l;
+    const int row = (int)__reduce_min_sync(full, in ? (uint32_t)c.row : 0xffffffffu);
+    src = __ffs((int)__ballot_sync(full, in && c.row == row)) - 1;
+  }
+  return Cand{h, __shfl_sync(full, c.l, src), __shfl_sync(full, c.row, src)};
+}
+// pivot_recip with the scaling by powers of two done on the exponent field; far exponents take the
+// general form (the same numbers, rounded at the same places)
+__device__ __forceinline__ cx<float> pivot_recip32(cx<float> a, int32_t* st) {
+  const uint32_t ex = __float_as_uint(fmaxf(fabsf(a.re), fabsf(a.im))) >> 23;  // no sign bit
+  if (ex < 64u || ex > 190u) return pivot_recip(a, st);
+  const float down = __uint_as_float((253u - ex) << 23);  // 2^(126 - ex): the larger part in [0.5, 1)
+  const float ar = __fmul_rn(a.re, down), ai = __fmul_rn(a.im, down);
+  const float inv = __fmul_rn(__frcp_rn(__fmaf_rn(ar, ar, __fmul_rn(ai, ai))), down);
+  return mkc<float>(__fmul_rn(ar, inv), __fmul_rn(-ai, inv));
+}
+
+constexpr int kPanelThreads = 512, kPanelWarps = kPanelThreads / 32;
+template <int W, int NR, bool LAST>
+__global__ void __launch_bounds__(kPanelThreads)
+    k_gj_panel32(int n, int k0, int w, int nb, const cx<float>* srcs, cx<float>* dsts,
+                 cx<float>* U, int32_t* piv, int32_t* conts, int32_t* status,
+                 const int32_t* active) {
+  const int p = blockIdx.x;
+  if (active && !active[p]) return;
+  constexpr int kG = kPanelThreads / W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  // slot NR - 1 holds the last rows: slot i of group g has row g + i kG - off, and the rows outside
+  // [0, n) are zeros that only fill the threads (every slot of every thread then does the same work,
+  // with no test that would part the slots' instructions)
+  const int off = (NR - 1 - n / kG) * kG;
+  cx<float>* fbuf = reinterpret_cast<cx<float>*>(smem_raw);  // [2][NR kG] pivot columns in turn
+  int* cont = reinterpret_cast<int*>(fbuf + 2 * NR * kG);    // [n]
+  const cx<float> zero = mkc<float>(0.0f, 0.0f);
+  __shared__ Cand best_of[kPanelWarps];
+  __shared__ cx<float> rowj[W], rowp[W], recip;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int c = tid % W, g = tid / W;
+  int32_t* st = status ? status + p : nullptr;
+  const long long nn = (long long)n * n;
+  const cx<float>* a = srcs + p * nn;
+  auto row_of = [&](int i) { return g + i * kG - off; };
+  // rows that an unrolling by four of steps of `old` rows leaves over: in a full panel such rows
+  // are in the last four slots
+  const int old = 256 / w;
+  auto left_over = [&](int r) { return r % old + (r / (4 * old) * 4 + 3) * old >= n; };
+  constexpr int kTail = LAST ? 0 : NR - 4;
+  unsigned long long other = 0;
+#pragma unroll
+  for (int i = kTail; i < NR; ++i)
+    if (row_of(i) >= 0 && left_over(row_of(i))) other |= 1ull << i;
+  cx<float> v[NR];
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int r = row_of(i);
+    v[i] = (r >= 0 && r < n && c < w) ? a[(long long)r * n + k0 + c] : zero;
+  }
+  for (int r = tid; r < n; r += kPanelThreads) cont[r] = r;
+  for (int jj = 0; jj < w; ++jj) {
+    const int j = k0 + jj;
+    cx<float>* slots = fbuf + (jj & 1) * NR * kG;  // the last step's column may still be read
+    cx<float>* f = slots + off;                    // by row
+    // the pivot column, and its largest entry in rows [j, n).  Its registers start the update from 0
+    if (c == jj) {
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        slots[g + i * kG] = v[i];
+        v[i] = zero;
+      }
+    }
+    __syncthreads();
+    const int w0 = n > kPanelThreads ? 0 : j / 32;  // first warp with a candidate
+    const int w1 = min(kPanelWarps, (n + 31) / 32);
+    if (wid >= w0 && wid < w1) {
+      Cand best{0u, 0u, n};
+      for (int r = tid; r < n; r += kPanelThreads) {
+        if (r < j) continue;
+        const Cand cand = candidate(f[r], r);
+        if (wins(cand, best)) best = cand;
+      }
+      best = warp_winner(best);
+      if (lane == 0) best_of[wid] = best;
+    }
+    __syncthreads();
+    // every warp combines the winners
+    const bool mine = lane >= w0 && lane < w1;
+    const Cand top = warp_winner(mine ? best_of[lane] : Cand{0u, 0u, n});
+    const int pr = top.row >= n ? j : top.row;
+    // rows j and pr go to shared memory
+    const int ij = (j + off) / kG, ip = (pr + off) / kG;
+    const bool own_j = j % kG == g, own_p = pr % kG == g;
+    if (own_j || own_p) {
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        if (own_j && i == ij) rowj[c] = v[i];
+        if (own_p && i == ip) rowp[c] = v[i];
+      }
+    }
+    if (tid == 0) {
+      recip = pivot_recip32(f[pr], st);
+      f[pr] = f[j];  // after the exchange row pr holds row j's old content
+      piv[(long long)p * n + j] = pr;
+      const int t = cont[j];
+      cont[j] = cont[pr];
+      cont[pr] = t;
+    }
+    __syncthreads();
+    const cx<float> d = recip;
+    const cx<float> pj = c == jj ? d : cmul(rowp[c], d);
+    if (own_p) {
+      const cx<float> moved = rowj[c];
+#pragma unroll
+      for (int i = 0; i < NR; ++i)
+        if (i == ip) v[i] = moved;
+    }
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+      eliminate(v[i], slots[g + i * kG], pj, i >= kTail && (other >> i & 1ull));
+    if (own_j) {
+#pragma unroll
+      for (int i = 0; i < NR; ++i)
+        if (i == ij) v[i] = pj;
+    }
+  }
+  __syncthreads();
+  cx<float>* o = dsts + p * nn;
+  cx<float>* u = U + (long long)p * n * nb;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int r = row_of(i);
+    if (r >= 0 && r < n && c < w) {
+      o[(long long)r * n + k0 + c] = v[i];
+      u[(long long)r * nb + c] = v[i];
+    }
+  }
+  for (int r = tid; r < n; r += kPanelThreads) conts[(long long)p * n + r] = cont[r];
+}
+
+// Trailing update of a panel step: dst = E src + U T outside the panel's columns, where E applies
+// the panel's row exchanges (row r of the result starts from row cont[r] of src) and clears the
+// pivot rows, U is the eliminated panel (n x w, row stride nb) and T the pivot rows
+// src[cont[k0 + k]].  An 80 x 80 block per CTA (n = 400 is 5 x 5 blocks with no padding; 64 x 64
+// blocks would pad it to 448^2, 25 % more work), each thread 5 x 5 complex accumulators: rows
+// ty + 16 i, columns tx + 16 j.  The whole U and T blocks are staged in shared memory at once (one
+// barrier), and src is read into the accumulators before the multiply-adds so that its latency
+// overlaps the staging.
 constexpr int kMaxPanel = 32;
 constexpr int kUpdTile = 80;
-template <typename R>
-__global__ void __launch_bounds__(256) k_gj_update(int n, int w, int nb, const cx<R>* U,
-                                                   const cx<R>* T, BM<R> C,
-                                                   const int32_t* active) {
+__global__ void __launch_bounds__(256) k_gj_update32(int n, int k0, int w, int nb,
+                                                     const cx<float>* U, const cx<float>* srcs,
+                                                     cx<float>* dsts, const int32_t* conts,
+                                                     const int32_t* active) {
   const int p = blockIdx.z;
   if (active && !active[p]) return;
-  __shared__ cx<R> Us[kUpdTile][kMaxPanel + 1];  // row-major like U; padded rows
-  __shared__ cx<R> Ts[kMaxPanel][kUpdTile];
+  __shared__ cx<float> Us[kUpdTile][kMaxPanel + 1];  // row-major like U; padded rows
+  __shared__ cx<float> Ts[kMaxPanel][kUpdTile];
   const int m0 = blockIdx.y * kUpdTile, n0 = blockIdx.x * kUpdTile;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const cx<R>* u = U + (long long)p * n * nb;
-  const cx<R>* t = T + (long long)p * nb * n;
-  cx<R>* c = bat(C, p);
-  const cx<R> zero = mkc<R>(R(0), R(0));
-  cx<R> acc[5][5];
+  const long long nn = (long long)n * n;
+  const cx<float>* u = U + (long long)p * n * nb;
+  const cx<float>* src = srcs + p * nn;
+  cx<float>* dst = dsts + p * nn;
+  const int32_t* cont = conts + (long long)p * n;
+  const cx<float> zero = mkc<float>(0.0f, 0.0f);
+  cx<float> acc[5][5];
 #pragma unroll
-  for (int i = 0; i < 5; ++i)
+  for (int i = 0; i < 5; ++i) {
+    const int r = m0 + ty + 16 * i;
+    const bool keep = r < n && (r < k0 || r >= k0 + w);
+    const cx<float>* row = src + (long long)(keep ? cont[r] : 0) * n;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-      const int r = m0 + ty + 16 * i, col = n0 + tx + 16 * j;
-      acc[i][j] = (r < n && col < n) ? c[(long long)r * C.ld + col] : zero;
+      const int col = n0 + tx + 16 * j;
+      acc[i][j] = (keep && col < n) ? row[col] : zero;
     }
+  }
   // staging: slot e of U is (row e / 32, column e % 32), of T (row e / 80, column e % 80); all
   // loads are issued before the first shared-memory store
   constexpr int kPer = kMaxPanel * kUpdTile / 256;  // 10
-  cx<R> us[kPer], ts[kPer];
+  cx<float> us[kPer], ts[kPer];
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
     const int e = threadIdx.x + 256 * q;
@@ -375,7 +576,7 @@ __global__ void __launch_bounds__(256) k_gj_update(int n, int w, int nb, const c
   for (int q = 0; q < kPer; ++q) {
     const int e = threadIdx.x + 256 * q;
     const int k = e / kUpdTile, col = e % kUpdTile;
-    ts[q] = (k < w && n0 + col < n) ? t[(long long)k * n + n0 + col] : zero;
+    ts[q] = (k < w && n0 + col < n) ? src[(long long)cont[k0 + k] * n + n0 + col] : zero;
   }
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
@@ -385,7 +586,7 @@ __global__ void __launch_bounds__(256) k_gj_update(int n, int w, int nb, const c
   }
   __syncthreads();
   for (int k = 0; k < w; ++k) {
-    cx<R> av[5], bv[5];
+    cx<float> av[5], bv[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) av[i] = Us[ty + 16 * i][k];
 #pragma unroll
@@ -400,34 +601,66 @@ __global__ void __launch_bounds__(256) k_gj_update(int n, int w, int nb, const c
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
       const int r = m0 + ty + 16 * i, col = n0 + tx + 16 * j;
-      if (r < n && col < n) c[(long long)r * C.ld + col] = acc[i][j];
+      if (r < n && col < n && (col < k0 || col >= k0 + w)) dst[(long long)r * n + col] = acc[i][j];
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_gj_unpermute(int n, BM<R> Am, BM<R> X,
-                                                           const int32_t* piv,
-                                                           const int32_t* active) {
+// Column permutation that the pivoting left: column c of the inverse is column map[c] of the
+// eliminated matrix.  A chain of exchanges, so one thread per item follows it in shared memory.
+__global__ void __launch_bounds__(kThreads) k_gj_perm(int n, const int32_t* piv, int32_t* map,
+                                                      const int32_t* active) {
   const int p = blockIdx.x;
   if (active && !active[p]) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int* src = reinterpret_cast<int*>(smem_raw);
-  const int32_t* pv = piv + (long long)p * n;
+  int* pv = src + n;
+  for (int c = threadIdx.x; c < n; c += blockDim.x) {
+    src[c] = c;
+    pv[c] = piv[(long long)p * n + c];
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    for (int c = 0; c < n; ++c) src[c] = c;
     for (int j = n - 1; j >= 0; --j) {
-      int t = src[j];
-      src[j] = src[pv[j]];
-      src[pv[j]] = t;
+      const int q = pv[j], t = src[j];
+      src[j] = src[q];
+      src[q] = t;
     }
   }
   __syncthreads();
-  const cx<R>* a = bat(Am, p);
-  cx<R>* x = bat(X, p);
-  for (long long e = threadIdx.x; e < (long long)n * n; e += blockDim.x) {
-    int r = (int)(e / n), c = (int)(e % n);
-    x[(long long)r * X.ld + c] = a[(long long)r * Am.ld + src[c]];
+  for (int c = threadIdx.x; c < n; c += blockDim.x) map[(long long)p * n + c] = src[c];
+}
+
+// X = the columns of A in their final order (A and X may differ in precision), one row at a time
+// per CTA through all CTAs of an item.
+template <typename RA, typename RX>
+__global__ void __launch_bounds__(kThreads) k_gj_columns(int n, BMc<RA> Am, BM<RX> Xm,
+                                                         const int32_t* map,
+                                                         const int32_t* active) {
+  const int p = blockIdx.y;
+  if (active && !active[p]) return;
+  const cx<RA>* a = bat(Am, p);
+  cx<RX>* x = bat(Xm, p);
+  const int32_t* m = map + (long long)p * n;
+  for (int r = blockIdx.x; r < n; r += gridDim.x)
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+      const cx<RA> v = a[(long long)r * Am.ld + m[c]];
+      x[(long long)r * Xm.ld + c] = mkc<RX>((RX)v.re, (RX)v.im);
+    }
+}
+
+// X = A and a change of precision (the one-CTA form's input and output)
+template <typename RA, typename RX>
+__global__ void __launch_bounds__(kThreads) k_convert(long long n, const cx<RA>* a, cx<RX>* x,
+                                                      const int32_t* active, long long per) {
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
+       k += (long long)gridDim.x * blockDim.x) {
+    if (active && !active[k / per]) continue;
+    x[k] = mkc<RX>((RX)a[k].re, (RX)a[k].im);
   }
+}
+inline unsigned convert_blocks(long long n) {
+  const long long b = (n + kThreads - 1) / kThreads;
+  return (unsigned)(b > 152 * 32 ? 152 * 32 : (b < 1 ? 1 : b));
 }
 
 }  // namespace
@@ -461,56 +694,132 @@ int gj_panel_width(int n, int elem_bytes) {
   return std::max(1, p2);
 }
 
-template <typename R>
-cudaError_t gj_inverse(cudaStream_t s, int P, int n, BM<R> M, BM<R> X, cx<R>* U, cx<R>* T,
-                       int32_t* piv, int32_t* status, const int32_t* active) {
+namespace {
+template <typename RA, typename RX>
+cudaError_t columns(cudaStream_t s, int P, int n, BMc<RA> A, BM<RX> X, const int32_t* piv,
+                    int32_t* map, const int32_t* active) {
+  static std::atomic<unsigned> attr{0};
+  cudaError_t e = set_smem_once(attr, reinterpret_cast<const void*>(&k_gj_perm), 96 * 1024);
+  if (e != cudaSuccess) return e;
+  k_gj_perm<<<P, kThreads, 2 * (size_t)n * sizeof(int), s>>>(n, piv, map, active);
+  k_gj_columns<RA, RX><<<dim3(std::min(n, 128), P), kThreads, 0, s>>>(n, A, X, map, active);
+  count_launch(2);
+  return cudaGetLastError();
+}
+
+template <int W, int NR, bool LAST>
+cudaError_t panel32(cudaStream_t s, int P, int n, int k0, int w, int nb, const cx<float>* src,
+                    cx<float>* dst, cx<float>* U, int32_t* piv, int32_t* cont, int32_t* status,
+                    const int32_t* active) {
+  static std::atomic<unsigned> attr{0};
+  auto* fn = &k_gj_panel32<W, NR, LAST>;
+  cudaError_t e = set_smem_once(attr, reinterpret_cast<const void*>(fn), 220 * 1024);
+  if (e != cudaSuccess) return e;
+  const size_t smem = 2 * (size_t)NR * (kPanelThreads / W) * sizeof(cx<float>) + n * sizeof(int);
+  fn<<<P, kPanelThreads, smem, s>>>(n, k0, w, nb, src, dst, U, piv, cont, status, active);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// The panel kernel of width nb, by the rows a thread holds (gj_panel_width keeps n nb <= 22528, so
+// n / kG + 1 <= 45; at nb = 1, n <= 9266 and 19).
+cudaError_t panel32(cudaStream_t s, int P, int n, int k0, int w, int nb, const cx<float>* src,
+                    cx<float>* dst, cx<float>* U, int32_t* piv, int32_t* cont, int32_t* status,
+                    const int32_t* active) {
+#define NEGF_PANEL_ARGS s, P, n, k0, w, nb, src, dst, U, piv, cont, status, active
+#define NEGF_PANEL(W_)                                                              \
+  case W_:                                                                          \
+    if (w < W_) return panel32<W_, 45, true>(NEGF_PANEL_ARGS);                      \
+    if (n * nb < 14 * kPanelThreads) return panel32<W_, 14, false>(NEGF_PANEL_ARGS); \
+    if (n * nb < 28 * kPanelThreads) return panel32<W_, 28, false>(NEGF_PANEL_ARGS); \
+    return panel32<W_, 45, false>(NEGF_PANEL_ARGS)
+  switch (nb) {
+    NEGF_PANEL(32);
+    NEGF_PANEL(16);
+    NEGF_PANEL(8);
+    NEGF_PANEL(4);
+    NEGF_PANEL(2);
+    case 1: return panel32<1, 19, false>(NEGF_PANEL_ARGS);
+  }
+#undef NEGF_PANEL
+#undef NEGF_PANEL_ARGS
+  return cudaErrorInvalidValue;
+}
+}  // namespace
+
+cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, z64* U, z64* T,
+                         int32_t* piv, int32_t* status, const int32_t* active) {
   if (P <= 0 || n <= 0) return cudaSuccess;
-  const int eb = (int)sizeof(cx<R>);
+  const int eb = (int)sizeof(z64);
   if (gj_fits_small(n, eb)) {
     size_t smem = small_smem(n, eb);
-    cudaError_t e = cudaFuncSetAttribute(k_gj_small<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_gj_small<double>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemBudget + 1024);
     if (e != cudaSuccess) return e;
-    k_gj_small<R><<<P, kThreads, smem, s>>>(n, M, X, status, active);
+    k_gj_small<double><<<P, kThreads, smem, s>>>(n, M, X, status, active);
     count_launch();
     return cudaGetLastError();
   }
   const int nb = gj_panel_width(n, eb);
-  cudaError_t e = cudaFuncSetAttribute(k_gj_panel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_gj_panel<double>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kSmemBudget + 1024);
   if (e != cudaSuccess) return e;
   for (int k0 = 0; k0 < n; k0 += nb) {
     const int w = std::min(nb, n - k0);
     size_t smem = panel_smem(n, w, eb);
     prof_begin(s, PROF_GJ_PANEL);
-    k_gj_panel<R><<<P, kThreads, smem, s>>>(n, k0, w, nb, M, U, T, piv, status, active);
+    k_gj_panel<double><<<P, kThreads, smem, s>>>(n, k0, w, nb, M, U, T, piv, status, active);
     prof_end(s, PROF_GJ_PANEL);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if constexpr (std::is_same<R, float>::value) {
-      // FP32: panels are at most kMaxPanel wide (gj_panel_width); FP64 is FMA-bound either way
-      k_gj_update<R><<<dim3((n + kUpdTile - 1) / kUpdTile, (n + kUpdTile - 1) / kUpdTile, P),
-                       256, 0, s>>>(n, w, nb, U, T, M, active);
-      count_launch();
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else {
-      BMc<R> Ua{U, (long long)n * nb, nullptr, nb};
-      BMc<R> Ta{T, (long long)nb * n, nullptr, n};
-      BMc<R> none{nullptr, 0, nullptr, 0};
-      e = gemm_simt<R>(s, P, n, n, w, mkc<double>(1.0, 0.0), Ua, OP_N, Ta, OP_N,
-                       mkc<double>(1.0, 0.0), M, mkc<double>(0.0, 0.0), none, active);
-      if (e != cudaSuccess) return e;
-    }
+    BMc<double> Ua{U, (long long)n * nb, nullptr, nb};
+    BMc<double> Ta{T, (long long)nb * n, nullptr, n};
+    BMc<double> none{nullptr, 0, nullptr, 0};
+    e = gemm_simt<double>(s, P, n, n, w, mkc<double>(1.0, 0.0), Ua, OP_N, Ta, OP_N,
+                          mkc<double>(1.0, 0.0), M, mkc<double>(0.0, 0.0), none, active);
+    if (e != cudaSuccess) return e;
   }
-  k_gj_unpermute<R><<<P, kThreads, n * sizeof(int), s>>>(n, M, X, piv, active);
-  count_launch();
-  return cudaGetLastError();
+  // T is free again
+  return columns<double, double>(s, P, n, cst(M), X, piv, reinterpret_cast<int32_t*>(T), active);
 }
 
-template cudaError_t gj_inverse<double>(cudaStream_t, int, int, BM<double>, BM<double>,
-                                        cx<double>*, cx<double>*, int32_t*, int32_t*,
-                                        const int32_t*);
-template cudaError_t gj_inverse<float>(cudaStream_t, int, int, BM<float>, BM<float>, cx<float>*,
-                                       cx<float>*, int32_t*, int32_t*, const int32_t*);
+cudaError_t gj_inverse32(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, cx<float>* m32,
+                         cx<float>* x32, cx<float>* U, int32_t* piv, int32_t* map, int32_t* status,
+                         const int32_t* active) {
+  if (P <= 0 || n <= 0) return cudaSuccess;
+  const int eb = (int)sizeof(cx<float>);
+  const long long nn = (long long)n * n, tot = P * nn;
+  k_convert<double, float><<<convert_blocks(tot), kThreads, 0, s>>>(tot, M.p, m32, active, nn);
+  count_launch();
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (gj_fits_small(n, eb)) {
+    e = cudaFuncSetAttribute(k_gj_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kSmemBudget + 1024);
+    if (e != cudaSuccess) return e;
+    k_gj_small<float><<<P, kThreads, small_smem(n, eb), s>>>(
+        n, BM<float>{m32, nn, nullptr, n}, BM<float>{x32, nn, nullptr, n}, status, active);
+    k_convert<float, double><<<convert_blocks(tot), kThreads, 0, s>>>(tot, x32, X.p, active, nn);
+    count_launch(2);
+    return cudaGetLastError();
+  }
+  const int nb = gj_panel_width(n, eb);
+  cx<float>*src = m32, *dst = x32;
+  const dim3 grid((n + kUpdTile - 1) / kUpdTile, (n + kUpdTile - 1) / kUpdTile, P);
+  for (int k0 = 0; k0 < n; k0 += nb) {
+    const int w = std::min(nb, n - k0);
+    prof_begin(s, PROF_GJ_PANEL);
+    e = panel32(s, P, n, k0, w, nb, src, dst, U, piv, map, status, active);
+    prof_end(s, PROF_GJ_PANEL);
+    if (e != cudaSuccess) return e;
+    k_gj_update32<<<grid, 256, 0, s>>>(n, k0, w, nb, U, src, dst, map, active);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    std::swap(src, dst);
+  }
+  return columns<float, double>(s, P, n, BMc<float>{src, nn, nullptr, n}, X, piv, map, active);
+}
 
 }  // namespace negf

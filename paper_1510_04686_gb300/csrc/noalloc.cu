@@ -61,7 +61,7 @@ extern "C" negf_status negf_zinv_batched_noalloc(int32_t n_batch, int32_t n, dou
   size_t off = 0;
   carve_engine(static_cast<char*>(base), off, n_batch, n, NEGF_PREC_FP64, false, w);
   const long long nn = (long long)n * n;
-  cudaError_t e = gj_inverse<double>(s, n_batch, n, BM<double>{reinterpret_cast<z64*>(M), nn, nullptr, n},
+  cudaError_t e = gj_inverse64(s, n_batch, n, BM<double>{reinterpret_cast<z64*>(M), nn, nullptr, n},
                                      BM<double>{reinterpret_cast<z64*>(X), nn, nullptr, n}, w.invU,
                                      w.invT, w.piv, status, nullptr);
   return e == cudaSuccess ? NEGF_OK : NEGF_ERR_CUDA;
