@@ -50,7 +50,7 @@ negf_status negf_zgemm_batched(int32_t precision, int32_t n_batch, int32_t M, in
   cudaError_t e;
   if (precision == NEGF_PREC_FP64) {
     if (K == 0) return NEGF_ERR_UNSUPPORTED;
-    e = gemm_simt<double>(s, n_batch, M, N, K, al, a, opA, b, opB, be, c, zero, none, nullptr);
+    e = gemm_simt(s, n_batch, M, N, K, al, a, opA, b, opB, be, c, zero, none, nullptr);
   } else {
     if (K == 0) return NEGF_ERR_UNSUPPORTED;
     size_t off = 0;

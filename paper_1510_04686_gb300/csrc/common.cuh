@@ -103,10 +103,9 @@ __device__ __forceinline__ cx<R>* bat(BM<R> a, int p) {
 // C[p] = alpha op(A[p]) op(B[p]) + beta C[p] + gamma D[p] on the CUDA cores (FP64 form).
 // beta == 0 does not read C; D.p == NULL skips the D term.  Batch items with
 // active[p] == 0 are skipped (active may be NULL).
-template <typename R>
-cudaError_t gemm_simt(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<R> A, int opA,
-                      BMc<R> B, int opB, z64 beta, BM<R> C, z64 gamma, BMc<R> D,
-                      const int32_t* active);
+cudaError_t gemm_simt(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
+                      int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
+                      BMc<double> D, const int32_t* active);
 
 // X[p] = M[p]^-1 by Gauss-Jordan elimination with partial pivoting (largest |m|, lowest row
 // on ties, pivots compared in FP64).  A zero pivot sets NEGF_PT_SINGULAR in status[p] and is

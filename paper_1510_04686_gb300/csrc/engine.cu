@@ -124,7 +124,7 @@ cudaError_t Engine::gemm(int P, int M, int N, int K, z64 alpha, BMc<double> A, i
   if (prec_mixed(prec))
     return tc_gemm(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, false, active,
                    tc_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys);
-  return gemm_simt<double>(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, active);
+  return gemm_simt(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, active);
 }
 
 cudaError_t Engine::timeout_reset() {

@@ -37,7 +37,10 @@ struct Mag {
 template <typename R>
 __device__ __forceinline__ Mag<R> mag2(cx<R> a) {
   if constexpr (sizeof(R) == 8) {
-    return Mag<R>{a.re * a.re + a.im * a.im, 0.0};
+    const double v = a.re * a.re + a.im * a.im;
+    // NaN, of either sign, gets a value that loses to every other one
+    const bool nan = (unsigned long long)__double_as_longlong(v) > 0x7ff0000000000000ull;
+    return Mag<R>{nan ? -0.5 : v, 0.0};
   } else {
     const float p = __fmul_rn(a.re, a.re), q = __fmul_rn(a.im, a.im);
     const float ep = fmaf(a.re, a.re, -p), eq = fmaf(a.im, a.im, -q);
@@ -51,8 +54,15 @@ __device__ __forceinline__ Mag<R> mag2(cx<R> a) {
 // (a.hi - b.hi) + (a.lo - b.lo) is that of the exact difference except within FP64-level ties.
 template <typename R>
 __device__ __forceinline__ bool better(Mag<R> a, int ia, Mag<R> b, int ib) {
-  const R d = (a.hi - b.hi) + (a.lo - b.lo);
-  return d > R(0) || (d == R(0) && ia < ib);
+  if constexpr (sizeof(R) == 8) {
+    // lo = 0; magnitudes order like their bit patterns (the start value -1 below all of them, the
+    // -0.5 for NaN below that), and integer comparisons leave the scarce FP64 pipe alone
+    const long long x = __double_as_longlong(a.hi), y = __double_as_longlong(b.hi);
+    return x > y || (x == y && ia < ib);
+  } else {
+    const R d = (a.hi - b.hi) + (a.lo - b.lo);
+    return d > R(0) || (d == R(0) && ia < ib);
+  }
 }
 
 // 1 / a, flagging an exactly zero pivot (replaced by a tiny number so the sweep goes on).  FP64
@@ -777,8 +787,8 @@ cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> 
     BMc<double> Ua{U, (long long)n * nb, nullptr, nb};
     BMc<double> Ta{T, (long long)nb * n, nullptr, n};
     BMc<double> none{nullptr, 0, nullptr, 0};
-    e = gemm_simt<double>(s, P, n, n, w, mkc<double>(1.0, 0.0), Ua, OP_N, Ta, OP_N,
-                          mkc<double>(1.0, 0.0), M, mkc<double>(0.0, 0.0), none, active);
+    e = gemm_simt(s, P, n, n, w, mkc<double>(1.0, 0.0), Ua, OP_N, Ta, OP_N, mkc<double>(1.0, 0.0),
+                  M, mkc<double>(0.0, 0.0), none, active);
     if (e != cudaSuccess) return e;
   }
   // T is free again
