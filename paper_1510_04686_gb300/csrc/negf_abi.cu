@@ -63,6 +63,7 @@ bool valid_opt(const negf_options* o) {
 struct LeadWs {
   z64 *eps_s, *eps, *al, *be, *al2, *be2, *g, *ag, *bg, *T1, *M;
   double* scale;
+  unsigned long long* top;  // largest entry of alpha, beta of each item (zero between steps)
   int32_t *active, *iters, *item_status, *n_active, *sys, *act_side;
   EngineWs eng;
 };
@@ -82,6 +83,7 @@ void carve_lead(Carver& c, int P, int b, bool res, const negf_options* opt, Lead
   w.T1 = c.take<z64>(Q * bb);
   w.M = c.take<z64>(Q * bb);
   w.scale = c.take<double>(Q);
+  w.top = c.take<unsigned long long>(Q);
   w.active = c.take<int32_t>(Q);
   w.iters = c.take<int32_t>(Q);
   w.item_status = c.take<int32_t>(Q);
@@ -95,6 +97,7 @@ struct RgfWs {
   int32_t *sys, *erow;
   z64 *g, *gl, *Lb;
   z64 *Y, *K, *Vt, *S, *W, *LW, *Gn, *Qm, *U, *Mt;
+  double* part;  // partial sums of the traces, 8 per point
   EngineWs eng;
 };
 
@@ -102,6 +105,7 @@ void carve_rgf(Carver& c, int P, int b, int N, bool res, const negf_options* opt
   const size_t bb = (size_t)b * b, PB = (size_t)P * bb;
   w.sys = c.take<int32_t>((size_t)P);
   w.erow = c.take<int32_t>((size_t)P);
+  w.part = c.take<double>(8 * (size_t)P);
   w.g = c.take<z64>((size_t)N * PB);
   w.gl = c.take<z64>((size_t)N * PB);
   w.Lb = c.take<z64>((size_t)std::max(N - 1, 1) * PB);
@@ -181,6 +185,7 @@ negf_status lead_chunk_run(const negf_device* dev, int P, bool res, const double
   BMc<double> Hu{reinterpret_cast<const z64*>(dev->H_up), (long long)((N - 1) * bb), sys, b};
   CK(launch_sr_init(s, Q, b, N, Hd, Hu, flat(w.eps_s, bb, b), flat(w.eps, bb, b),
                     flat(w.al, bb, b), flat(w.be, bb, b), w.scale));
+  CK(cudaMemsetAsync(w.top, 0, (size_t)Q * sizeof(unsigned long long), s));
   CK(launch_fill_i32(s, w.active, Q, 1));
   CK(launch_fill_i32(s, w.iters, Q, 0));
   CK(launch_fill_i32(s, w.item_status, Q, 0));
@@ -258,7 +263,7 @@ negf_status lead_chunk_run(const negf_device* dev, int P, bool res, const double
     std::swap(be, be2);
     CK(cudaMemsetAsync(w.n_active, 0, sizeof(int32_t), s));
     CK(launch_sr_check(s, Q, b, it, opt->sr_tol, cst(flat(al, bb, b)), cst(flat(be, bb, b)),
-                       w.scale, w.active, w.iters, w.n_active, iface ? w.act_side : nullptr));
+                       w.scale, w.active, w.iters, w.n_active, iface ? w.act_side : nullptr, w.top));
     const int chk = opt->sr_host_check;
     if (chk > 0 && it >= 8 && (it % chk == 0 || it == opt->sr_max_iter)) {
       CK(cudaMemcpyAsync(&h_active, w.n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -454,7 +459,7 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
     CK(eng.gemm(P, b, b, b, one, Fc(G[N - 1]), OP_N, Fc(w.S), OP_N, zero, F(w.LW), zero, kNone,
                 nullptr));
     CK(launch_transmission(s, P, b, Fc(w.S), Fc(G[N - 1]), Fc(w.W), Fc(w.LW), a.transmission,
-                           nullptr));
+                           w.part, reinterpret_cast<double*>(w.Mt)));
   }
   CK(launch_slab_obs(s, P, b, N - 1, NB, a.A, Fc(G[N - 1]), Fc(GL[N - 1]), a.density, a.dGR,
                      a.dGL,
@@ -480,7 +485,8 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
     CK(eng.gemm(P, b, b, ir, two, cview(Fc(w.W), b - ir), OP_N, rview(Fc(GL[i]), b - ir), OP_N,
                 zero, F(w.U), one, Fc(w.Qm), nullptr));
     if (a.current)
-      CK(launch_bond_current(s, P, b, Hu(i), Fc(w.U), Fc(w.Qm), a.current + i, N - 1, nullptr));
+      CK(launch_bond_current(s, P, b, Hu(i), Fc(w.U), Fc(w.Qm), a.current + i, N - 1, w.part,
+                             reinterpret_cast<double*>(w.Mt)));  // Mt is written below
     // G^<_ii = AH(g^<_i + L U)  (interface mode: L[:, C] U[C, :])
     CK(eng.gemm(P, b, b, ic, one, Fc(L), OP_N, Fc(w.U), OP_N, zero, F(w.Mt), one, Fc(GL[i]),
                 nullptr));

@@ -10,17 +10,16 @@ namespace {
 constexpr int kT = 256;
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  double r = 0.0;
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r += sh[k];  // fixed order
+// Row and column of entry k of a matrix of b columns.  A 64-bit division costs several times a 32-bit
+// one, enough to hold up the kernels here, which otherwise move bytes.
+__device__ __forceinline__ void row_col(long long k, int b, int& r, int& c) {
+  if (k <= 0xffffffffll) {
+    r = (int)((unsigned)k / (unsigned)b);
+    c = (int)((unsigned)k - (unsigned)r * (unsigned)b);
+  } else {
+    r = (int)(k / b);
+    c = (int)(k % b);
   }
-  return r;
 }
 
 __device__ __forceinline__ double block_max(double v, double* sh) {
@@ -55,7 +54,8 @@ __global__ void k_assemble(int b, const double* E, double eta, BMc<double> Hd, c
   const double e = E[p];
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
        k += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
+    int r, c;
+    row_col(k, b, r, c);
     z64 v = mkc<double>(0.0, 0.0) - h[(long long)r * Hd.ld + c];
     if (r == c) {
       v.re += e - (V ? V[r] : 0.0);
@@ -80,7 +80,8 @@ __global__ void k_source(int b, const z64* scat, long long scat_stride, int A,
   z64* s = bat(S, p);
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
        k += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
+    int r, c;
+    row_col(k, b, r, c);
     z64 v = mkc<double>(0.0, 0.0);
     if (sa) v = v + sa[(long long)r * SigA.ld + c];
     if (sb) v = v + sb[(long long)r * SigB.ld + c];
@@ -96,7 +97,8 @@ __global__ void k_antiherm(int b, BMc<double> S, BM<double> O, const int32_t* ac
   z64* o = bat(O, p);
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
        k += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
+    int r, c;
+    row_col(k, b, r, c);
     z64 a = s[(long long)r * S.ld + c], t = s[(long long)c * S.ld + r];
     o[(long long)r * O.ld + c] = mkc<double>(0.5 * (a.re - t.re), 0.5 * (a.im + t.im));
   }
@@ -122,24 +124,84 @@ __global__ void k_slab_obs(int b, int i, int nb_tot, int A, BMc<double> G, BMc<d
   }
 }
 
+// The two traces below are sums over all b^2 entries of an item, in an order that has always been
+// that of one CTA of kT threads going through them row by row: thread t takes entries t, t + kT, ...,
+// then the threads of a warp are summed, then the warps in turn.  They keep it.  One factor is read
+// transposed, so the terms are formed first, tile by tile with every access in whole lines, and then
+// added by one CTA per such warp and item.  64 items of b = 400, bond current: 160 us (446 us with
+// one CTA per item doing both), against 72 us for its bytes.
+constexpr int kSumWarps = kT / 32;
+constexpr int kSumLoads = 16;  // entries in flight per thread
+constexpr int kTile = 32;
+__device__ __forceinline__ void warp_part(double v, double* part, int p) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  if (threadIdx.x == 0) part[p * kSumWarps + blockIdx.x] = v;
+}
+// terms: b^2 per item, or b^2 pairs of which the first is added and the second subtracted
+template <bool PAIRS>
+__global__ void __launch_bounds__(32) k_sum_terms(long long n, const double* terms, double* part) {
+  const double* v = terms + (long long)blockIdx.y * n * (PAIRS ? 2 : 1);
+  double acc = 0.0;
+  for (long long k0 = blockIdx.x * 32 + threadIdx.x; k0 < n; k0 += kSumLoads * kT) {
+    double x[kSumLoads], y[kSumLoads];
+#pragma unroll
+    for (int i = 0; i < kSumLoads; ++i) {
+      const long long k = k0 + i * kT;
+      if (PAIRS && k < n) {
+        const double2 t = reinterpret_cast<const double2*>(v)[k];
+        x[i] = t.x;
+        y[i] = t.y;
+      } else if (k < n) {
+        x[i] = v[k];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kSumLoads; ++i)
+      if (k0 + i * kT < n) {
+        acc += x[i];
+        if (PAIRS) acc -= y[i];
+      }
+  }
+  warp_part(acc, part, blockIdx.y);
+}
+// out[p] = the parts of item p in turn
+__global__ void k_sum_parts(int P, const double* part, double* out, long long out_stride) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= P) return;
+  double r = 0.0;
+  for (int k = 0; k < kSumWarps; ++k) r += part[p * kSumWarps + k];
+  out[p * out_stride] = r;
+}
+
+// Runs f(r, c, x^T[r][c]) over a tile of kTile^2 entries with threadIdx.x along c, x(r, c) being
+// read with threadIdx.x along its own columns
+template <typename X, typename F>
+__device__ __forceinline__ void transposed_tile(int b, X x, F f) {
+  __shared__ z64 tile[kTile][kTile + 1];
+  const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
+#pragma unroll
+  for (int i = threadIdx.y; i < kTile; i += 8)
+    if (c0 + i < b && r0 + threadIdx.x < b) tile[i][threadIdx.x] = x(c0 + i, r0 + threadIdx.x);
+  __syncthreads();
+#pragma unroll
+  for (int i = threadIdx.y; i < kTile; i += 8)
+    if (r0 + i < b && c0 + threadIdx.x < b) f(r0 + i, c0 + threadIdx.x, tile[threadIdx.x][i]);
+}
+
 // j_i = 2 Re Tr[t G^<_{i+1,i}] with G^<_{i+1,i} = (U + Q) / 2  ->  Re Tr[t (U + Q)]
-__global__ void k_bond_current(int b, BMc<double> Tm, BMc<double> U, BMc<double> Q, double* out,
-                               long long out_stride, const int32_t* active) {
-  const int p = blockIdx.x;
-  if (active && !active[p]) return;
-  __shared__ double sh[32];
+__global__ void __launch_bounds__(256) k_bond_terms(int b, BMc<double> Tm, BMc<double> U,
+                                                    BMc<double> Q, double* terms) {
+  const int p = blockIdx.z;
   const z64* t = bat(Tm, p);
   const z64* u = bat(U, p);
   const z64* q = bat(Q, p);
-  double acc = 0.0;
-  for (long long k = threadIdx.x; k < (long long)b * b; k += blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
-    z64 tv = t[(long long)r * Tm.ld + c];
-    z64 x = u[(long long)c * U.ld + r] + q[(long long)c * Q.ld + r];
-    acc += tv.re * x.re - tv.im * x.im;
-  }
-  double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) out[(long long)p * out_stride] = s;
+  double* out = terms + (long long)p * b * b;
+  transposed_tile(
+      b, [&](int r, int c) { return u[(long long)r * U.ld + c] + q[(long long)r * Q.ld + c]; },
+      [&](int r, int c, z64 x) {
+        const z64 tv = t[(long long)r * Tm.ld + c];
+        out[(long long)r * b + c] = tv.re * x.re - tv.im * x.im;
+      });
 }
 
 __global__ void k_gamma(int b, BMc<double> Sig, BM<double> Gam, const int32_t* active) {
@@ -149,7 +211,8 @@ __global__ void k_gamma(int b, BMc<double> Sig, BM<double> Gam, const int32_t* a
   z64* g = bat(Gam, p);
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
        k += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
+    int r, c;
+    row_col(k, b, r, c);
     z64 a = s[(long long)r * Sig.ld + c], t = s[(long long)c * Sig.ld + r];
     // i (a - conj(t))
     g[(long long)r * Gam.ld + c] = mkc<double>(-(a.im + t.im), a.re - t.re);
@@ -157,30 +220,37 @@ __global__ void k_gamma(int b, BMc<double> Sig, BM<double> Gam, const int32_t* a
 }
 
 // T = Re{ Tr[Gamma A] - sum_jk Y_jk conj(Z_jk) },  A = i (G - G^H), Y = Gamma G, Z = G Gamma
-__global__ void k_transmission(int b, BMc<double> Gam, BMc<double> G, BMc<double> Y,
-                               BMc<double> Z, double* out, const int32_t* active) {
-  const int p = blockIdx.x;
-  if (active && !active[p]) return;
-  __shared__ double sh[32];
+__global__ void __launch_bounds__(256) k_transmission_terms(int b, BMc<double> Gam, BMc<double> G,
+                                                            BMc<double> Y, BMc<double> Z,
+                                                            double* terms) {
+  const int p = blockIdx.z;
   const z64* gm = bat(Gam, p);
   const z64* g = bat(G, p);
   const z64* y = bat(Y, p);
   const z64* z = bat(Z, p);
-  double acc = 0.0;
-  for (long long k = threadIdx.x; k < (long long)b * b; k += blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
-    z64 gg = gm[(long long)r * Gam.ld + c];
-    z64 a1 = g[(long long)c * G.ld + r], a2 = g[(long long)r * G.ld + c];
-    // A_cr = i (G_cr - conj(G_rc))
-    z64 A = mkc<double>(-(a1.im + a2.im), a1.re - a2.re);
-    acc += gg.re * A.re - gg.im * A.im;
-    z64 yv = y[(long long)r * Y.ld + c], zv = z[(long long)r * Z.ld + c];
-    acc -= yv.re * zv.re + yv.im * zv.im;
-  }
-  double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) out[p] = s;
+  double* out = terms + (long long)p * b * b * 2;
+  transposed_tile(
+      b, [&](int r, int c) { return g[(long long)r * G.ld + c]; },
+      [&](int r, int c, z64 a1) {
+        const z64 gg = gm[(long long)r * Gam.ld + c], a2 = g[(long long)r * G.ld + c];
+        // A_cr = i (G_cr - conj(G_rc))
+        const z64 A = mkc<double>(-(a1.im + a2.im), a1.re - a2.re);
+        const z64 yv = y[(long long)r * Y.ld + c], zv = z[(long long)r * Z.ld + c];
+        double2 t;
+        t.x = gg.re * A.re - gg.im * A.im;
+        t.y = yv.re * zv.re + yv.im * zv.im;
+        reinterpret_cast<double2*>(out)[(long long)r * b + c] = t;
+      });
 }
 
+// Largest |v| of a CTA raised into *top (bit patterns of non-negative doubles order like the values;
+// NaN is passed over)
+__device__ __forceinline__ void raise_max(double v, double* sh, unsigned long long* top) {
+  const double m = block_max(v, sh);
+  if (threadIdx.x == 0 && m > 0.0) atomicMax(top, (unsigned long long)__double_as_longlong(m));
+}
+
+// scale: zeroed; raised to the largest entry of h and tau (k_sr_check takes 1 for 0)
 __global__ void k_sr_init(int b, int N, BMc<double> Hd, BMc<double> Hu, BM<double> eps_s,
                           BM<double> eps, BM<double> al, BM<double> be, double* scale) {
   // batch item q = 2 p + side; Hd / Hu batch addressing already per point (index p)
@@ -195,8 +265,10 @@ __global__ void k_sr_init(int b, int N, BMc<double> Hd, BMc<double> Hu, BM<doubl
   z64* a = bat(al, q);
   z64* bb = bat(be, q);
   double mx = 0.0;
-  for (long long k = threadIdx.x; k < (long long)b * b; k += blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
+       k += (long long)gridDim.x * blockDim.x) {
+    int r, c;
+    row_col(k, b, r, c);
     z64 hv = hd[k];
     es[k] = hv;
     e[k] = hv;
@@ -209,8 +281,7 @@ __global__ void k_sr_init(int b, int N, BMc<double> Hd, BMc<double> Hu, BM<doubl
     bb[k] = bv;
     mx = fmax(mx, fmax(fmax(fabs(hv.re), fabs(hv.im)), fmax(fabs(av.re), fabs(av.im))));
   }
-  double m = block_max(mx, sh);
-  if (threadIdx.x == 0) scale[q] = m > 0.0 ? m : 1.0;
+  raise_max(mx, sh, reinterpret_cast<unsigned long long*>(scale + q));
 }
 
 __global__ void k_zminus(int b, const double* E, double eta, BMc<double> X, BM<double> M,
@@ -222,7 +293,8 @@ __global__ void k_zminus(int b, const double* E, double eta, BMc<double> X, BM<d
   const double e = E[q >> 1];
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
        k += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(k / b), c = (int)(k % b);
+    int r, c;
+    row_col(k, b, r, c);
     z64 v = mkc<double>(0.0, 0.0) - x[k];
     if (r == c) {
       v.re += e;
@@ -251,29 +323,38 @@ __global__ void k_add2(int b, BMc<double> T1, BM<double> A1, BM<double> A2, int 
   }
 }
 
-__global__ void k_sr_check(int b, int it, double tol, BMc<double> al, BMc<double> be,
-                           const double* scale, int32_t* active, int32_t* iters,
-                           int32_t* n_active, int32_t* by_side) {
-  const int q = blockIdx.x;
+// top[q] (zero between steps) raised to the largest entry of alpha and beta
+__global__ void k_sr_max(int b, BMc<double> al, BMc<double> be, const int32_t* active,
+                         unsigned long long* top) {
+  const int q = blockIdx.y;
   if (!active[q]) return;
   __shared__ double sh[32];
   const z64* a = bat(al, q);
   const z64* c = bat(be, q);
   double mx = 0.0;
-  for (long long k = threadIdx.x; k < (long long)b * b; k += blockDim.x) {
+#pragma unroll 4
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)b * b;
+       k += (long long)gridDim.x * blockDim.x) {
     z64 u = a[k], v = c[k];
     mx = fmax(mx, fmax(fmax(fabs(u.re), fabs(u.im)), fmax(fabs(v.re), fabs(v.im))));
   }
-  double m = block_max(mx, sh);
-  if (threadIdx.x == 0) {
-    if (m < tol * scale[q]) {
-      active[q] = 0;
-      iters[q] = it;
-      // per-side copy of the mask: by_side[side * P + p] for q = 2 p + side
-      if (by_side) by_side[(q & 1) * (gridDim.x >> 1) + (q >> 1)] = 0;
-    } else {
-      atomicAdd(n_active, 1);
-    }
+  raise_max(mx, sh, top + q);
+}
+
+__global__ void k_sr_check(int Q, int it, double tol, const double* scale, int32_t* active,
+                           int32_t* iters, int32_t* n_active, int32_t* by_side,
+                           unsigned long long* top) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= Q || !active[q]) return;
+  const double m = __longlong_as_double((long long)top[q]);
+  top[q] = 0ull;
+  if (m < tol * (scale[q] > 0.0 ? scale[q] : 1.0)) {
+    active[q] = 0;
+    iters[q] = it;
+    // per-side copy of the mask: by_side[side * P + p] for q = 2 p + side
+    if (by_side) by_side[(q & 1) * (Q >> 1) + (q >> 1)] = 0;
+  } else {
+    atomicAdd(n_active, 1);
   }
 }
 
@@ -390,11 +471,20 @@ cudaError_t launch_slab_obs(cudaStream_t s, int P, int b, int i, int nb_tot, int
   count_launch();
   return cudaGetLastError();
 }
+namespace {
+// Tiles of b x b for P items, kTile^2 each; grid z holds at most 65535 items, as the products do.
+dim3 tile_grid(int b, int P) {
+  return dim3((b + kTile - 1) / kTile, (b + kTile - 1) / kTile, P);
+}
+}  // namespace
+
 cudaError_t launch_bond_current(cudaStream_t s, int P, int b, BMc<double> Tm, BMc<double> U,
-                                BMc<double> Q, double* out, long long out_stride,
-                                const int32_t* active) {
-  k_bond_current<<<P, kT, 0, s>>>(b, Tm, U, Q, out, out_stride, active);
-  count_launch();
+                                BMc<double> Q, double* out, long long out_stride, double* part,
+                                double* terms) {
+  k_bond_terms<<<tile_grid(b, P), dim3(kTile, 8), 0, s>>>(b, Tm, U, Q, terms);
+  k_sum_terms<false><<<dim3(kSumWarps, P), 32, 0, s>>>((long long)b * b, terms, part);
+  k_sum_parts<<<(P + kT - 1) / kT, kT, 0, s>>>(P, part, out, out_stride);
+  count_launch(3);
   return cudaGetLastError();
 }
 cudaError_t launch_gamma(cudaStream_t s, int P, int b, BMc<double> Sig, BM<double> Gam,
@@ -404,16 +494,20 @@ cudaError_t launch_gamma(cudaStream_t s, int P, int b, BMc<double> Sig, BM<doubl
   return cudaGetLastError();
 }
 cudaError_t launch_transmission(cudaStream_t s, int P, int b, BMc<double> Gam, BMc<double> G,
-                                BMc<double> Y, BMc<double> Z, double* out,
-                                const int32_t* active) {
-  k_transmission<<<P, kT, 0, s>>>(b, Gam, G, Y, Z, out, active);
-  count_launch();
+                                BMc<double> Y, BMc<double> Z, double* out, double* part,
+                                double* terms) {
+  k_transmission_terms<<<tile_grid(b, P), dim3(kTile, 8), 0, s>>>(b, Gam, G, Y, Z, terms);
+  k_sum_terms<true><<<dim3(kSumWarps, P), 32, 0, s>>>((long long)b * b, terms, part);
+  k_sum_parts<<<(P + kT - 1) / kT, kT, 0, s>>>(P, part, out, 1);
+  count_launch(3);
   return cudaGetLastError();
 }
 cudaError_t launch_sr_init(cudaStream_t s, int P2, int b, int N, BMc<double> Hd, BMc<double> Hu,
                            BM<double> eps_s, BM<double> eps, BM<double> al, BM<double> be,
                            double* scale) {
-  k_sr_init<<<dim3(1, P2), kT, 0, s>>>(b, N, Hd, Hu, eps_s, eps, al, be, scale);
+  cudaError_t e = cudaMemsetAsync(scale, 0, (size_t)P2 * sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  k_sr_init<<<grid2((long long)b * b, P2), kT, 0, s>>>(b, N, Hd, Hu, eps_s, eps, al, be, scale);
   count_launch();
   return cudaGetLastError();
 }
@@ -432,9 +526,13 @@ cudaError_t launch_add2(cudaStream_t s, int P2, int b, BMc<double> T1, BM<double
 }
 cudaError_t launch_sr_check(cudaStream_t s, int P2, int b, int it, double tol, BMc<double> al,
                             BMc<double> be, const double* scale, int32_t* active,
-                            int32_t* iters, int32_t* n_active, int32_t* by_side) {
-  k_sr_check<<<P2, kT, 0, s>>>(b, it, tol, al, be, scale, active, iters, n_active, by_side);
-  count_launch();
+                            int32_t* iters, int32_t* n_active, int32_t* by_side,
+                            unsigned long long* top) {
+  // many CTAs per item: with one, the maxima of 32 items of b = 400 took 300 us
+  k_sr_max<<<grid2((long long)b * b / 8, P2), kT, 0, s>>>(b, al, be, active, top);
+  k_sr_check<<<(P2 + kT - 1) / kT, kT, 0, s>>>(P2, it, tol, scale, active, iters, n_active, by_side,
+                                               top);
+  count_launch(2);
   return cudaGetLastError();
 }
 cudaError_t launch_lead_lesser(cudaStream_t s, int P2, int b, const double* E, double mu_L,

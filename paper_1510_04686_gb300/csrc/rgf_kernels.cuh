@@ -21,14 +21,15 @@ cudaError_t launch_antiherm(cudaStream_t s, int P, int b, BMc<double> S, BM<doub
 cudaError_t launch_slab_obs(cudaStream_t s, int P, int b, int i, int nb_tot, int A,
                             BMc<double> G, BMc<double> GL, double* density, z64* dGR, z64* dGL,
                             const int32_t* active);
+// part: scratch of 8 doubles per item; terms: of b^2 doubles per item (transmission: 2 b^2)
 cudaError_t launch_bond_current(cudaStream_t s, int P, int b, BMc<double> Tm, BMc<double> U,
-                                BMc<double> Q, double* out, long long out_stride,
-                                const int32_t* active);
+                                BMc<double> Q, double* out, long long out_stride, double* part,
+                                double* terms);
 cudaError_t launch_gamma(cudaStream_t s, int P, int b, BMc<double> Sig, BM<double> Gam,
                          const int32_t* active);
 cudaError_t launch_transmission(cudaStream_t s, int P, int b, BMc<double> Gam, BMc<double> G,
-                                BMc<double> Y, BMc<double> Z, double* out,
-                                const int32_t* active);
+                                BMc<double> Y, BMc<double> Z, double* out, double* part,
+                                double* terms);
 cudaError_t launch_sr_init(cudaStream_t s, int P2, int b, int N, BMc<double> Hd, BMc<double> Hu,
                            BM<double> eps_s, BM<double> eps, BM<double> al, BM<double> be,
                            double* scale);
@@ -41,7 +42,8 @@ cudaError_t launch_add2(cudaStream_t s, int P2, int b, BMc<double> T1, BM<double
 // by_side (nullable, [2][P2 / 2]): items that converge also clear by_side[side][p], q = 2 p + side.
 cudaError_t launch_sr_check(cudaStream_t s, int P2, int b, int it, double tol, BMc<double> al,
                             BMc<double> be, const double* scale, int32_t* active,
-                            int32_t* iters, int32_t* n_active, int32_t* by_side);
+                            int32_t* iters, int32_t* n_active, int32_t* by_side,
+                            unsigned long long* top);
 cudaError_t launch_lead_lesser(cudaStream_t s, int P2, int b, const double* E, double mu_L,
                                double mu_R, double kT_, BMc<double> Gam, BM<double> Les);
 cudaError_t launch_sr_status(cudaStream_t s, int P, const int32_t* active,
