@@ -83,14 +83,20 @@ __global__ void __launch_bounds__(256)
         Rdn = R0;
         Ldn = L0;
       }
-      // Eq. (4) acoustic, Eq. (6) optical retarded, Eq. (5) optical lesser
-      z64 nR, nL;
-      nR.re = D_ac * R0.re + D_op * ((1.0 + n0) * Rdn.re + n0 * Rup.re + 0.5 * Ldn.re - 0.5 * Lup.re);
-      nR.im = D_ac * R0.im + D_op * ((1.0 + n0) * Rdn.im + n0 * Rup.im + 0.5 * Ldn.im - 0.5 * Lup.im);
-      nL.re = D_ac * L0.re + D_op * ((1.0 + n0) * Lup.re + n0 * Ldn.re);
-      nL.im = D_ac * L0.im + D_op * ((1.0 + n0) * Lup.im + n0 * Ldn.im);
-      const z64 wR = mkc((1.0 - mix) * oR.re + mix * nR.re, (1.0 - mix) * oR.im + mix * nR.im);
-      const z64 wL = mkc((1.0 - mix) * oL.re + mix * nL.re, (1.0 - mix) * oL.im + mix * nL.im);
+      // Eq. (4) acoustic, Eq. (6) optical retarded, Eq. (5) optical lesser.  Which product of a sum
+      // is rounded before the addition is written out: left to the compiler, the last digit of the
+      // result changes with the code around it.
+      auto retarded = [&](double c, double dn, double up, double ldn, double lup, double old) {
+        const double g = fma(-0.5, lup, fma(0.5, ldn, fma(n0, up, (1.0 + n0) * dn)));
+        return fma(1.0 - mix, old, mix * fma(D_ac, c, D_op * g));
+      };
+      auto lesser = [&](double c, double dn, double up) {
+        return fma(D_ac, c, D_op * fma(1.0 + n0, up, n0 * dn));
+      };
+      const z64 wR = mkc(retarded(R0.re, Rdn.re, Rup.re, Ldn.re, Lup.re, oR.re),
+                         retarded(R0.im, Rdn.im, Rup.im, Ldn.im, Lup.im, oR.im));
+      const z64 wL = mkc(fma(1.0 - mix, oL.re, mix * lesser(L0.re, Ldn.re, Lup.re)),
+                         fma(mix, lesser(L0.im, Ldn.im, Lup.im), (1.0 - mix) * oL.im));
       top.add(wR, oR);
       top.add(wL, oL);
       sR[at] = wR;
