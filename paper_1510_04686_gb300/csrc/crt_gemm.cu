@@ -651,7 +651,11 @@ static int most_moduli(int K, int bits) {
 }
 
 void crt_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits, CrtWs& w) {
-  const size_t n = (size_t)most_moduli(K, bits), L = (size_t)residue_ld(K);
+  // a product may take a narrower tier than the one that the scratch is for
+  int most = 0;
+  for (int t : {40, 48, 56})
+    if (t <= bits) most = std::max(most, most_moduli(K, t));
+  const size_t n = (size_t)most, L = (size_t)residue_ld(K);
   auto take = [&](size_t bytes) -> void* {
     size_t a = (off + 1023) & ~size_t(1023);
     off = a + bytes;

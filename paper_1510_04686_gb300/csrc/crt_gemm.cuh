@@ -39,7 +39,7 @@ cudaError_t crt_prof_reset();
 
 // n_distinct: number of different matrices an indexed operand (idx != NULL) selects from
 // (0 = unknown: convert every item).  bits: fixed-point bits per operand value (tc_bits_ok); the
-// workspace must have been carved for the same bits.  rmax (nullable, float [P], zeroed by the
+// workspace must have been carved for these bits or more.  rmax (nullable, float [P], zeroed by the
 // caller): rmax[p] is raised to the largest |Re| or |Im| of item p's outputs (the Newton-Schulz
 // residual norm when C = I - M X).
 cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
