@@ -671,7 +671,7 @@ void crt_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits,
 cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
                     int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
                     BMc<double> D, bool add_identity, const int32_t* active, const CrtWs& ws,
-                    int bits, int n_distinct, float* rmax) {
+                    int bits, int n_distinct, float* rmax, Kept* kept) {
   if (P <= 0 || M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   // Operands shared by all items (stride 0) or selected per item from n_distinct matrices are
   // converted once per distinct matrix; the kernel maps each item to its residue set.
@@ -701,18 +701,27 @@ cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<
   const int L = residue_ld(K);
   __nv_bfloat16* ra = static_cast<__nv_bfloat16*>(ws.resA);
   __nv_bfloat16* rb = static_cast<__nv_bfloat16*>(ws.resB);
+  const KeptOperand ka{A.p,  ra,  g.zA ? g.zA : A.idx, actA, A.stride,   A.ld,
+                       opA, M, K, PA, g.plan.cls, 2 * g.plan.n + g.plan.hp};
+  const KeptOperand kb{B.p,  rb,  g.zB ? g.zB : B.idx, actB, B.stride,   B.ld,
+                       opB, N, K, PB, g.plan.cls, 2 * g.plan.n + g.plan.hp};
+  const bool haveA = kept && (kept->reuse & REUSE_A) && kept->a == ka;
+  const bool haveB = kept && (kept->reuse & REUSE_B) && kept->b == kb;
   prof_begin(s, PROF_SLICE);
   // a row of op(A) is a column of A in memory for op T/C; a column of op(B) is a column of B for
   // op N
-  cudaError_t e = launch_residues(s, g.plan, g.plan.alpha_a, g.plan.hp ? 1.0 : crt_const(g.plan).sigma, PA, M, K,
-                                  L, A, opA, opA != OP_N, ra,
-                                  ws.expA, actA);
+  cudaError_t e = cudaSuccess;
+  if (!haveA)
+    e = launch_residues(s, g.plan, g.plan.alpha_a, g.plan.hp ? 1.0 : crt_const(g.plan).sigma, PA, M,
+                        K, L, A, opA, opA != OP_N, ra, ws.expA, actA);
   if (e != cudaSuccess) return e;
-  e = launch_residues(s, g.plan, g.plan.alpha_b, 1.0, PB, N, K, L, B, opB, opB == OP_N, rb, ws.expB,
-                      actB);
+  if (!haveB)
+    e = launch_residues(s, g.plan, g.plan.alpha_b, 1.0, PB, N, K, L, B, opB, opB == OP_N, rb,
+                        ws.expB, actB);
   prof_end(s, PROF_SLICE);
-  count_launch(2);
+  count_launch(!haveA + !haveB);
   if (e != cudaSuccess) return e;
+  if (kept) *kept = Kept{ka, kb, 0};
   // the 56-bit tier's fractions carry correction sums, whose registers limit the tile to 64
   const bool hp = g.plan.hp;
   const int nt = pick_width(P, M, N, hp);

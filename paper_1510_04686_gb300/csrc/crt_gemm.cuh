@@ -15,6 +15,7 @@
 #pragma once
 #include "common.cuh"
 #include "crt_plan.cuh"
+#include "tc_gemm.cuh"
 
 namespace negf {
 
@@ -41,10 +42,10 @@ cudaError_t crt_prof_reset();
 // (0 = unknown: convert every item).  bits: fixed-point bits per operand value (tc_bits_ok); the
 // workspace must have been carved for these bits or more.  rmax (nullable, float [P], zeroed by the
 // caller): rmax[p] is raised to the largest |Re| or |Im| of item p's outputs (the Newton-Schulz
-// residual norm when C = I - M X).
+// residual norm when C = I - M X).  kept (nullable): what the scratch of `ws` holds, see Kept.
 cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
                     int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
                     BMc<double> D, bool add_identity, const int32_t* active, const CrtWs& ws,
-                    int bits, int n_distinct = 0, float* rmax = nullptr);
+                    int bits, int n_distinct = 0, float* rmax = nullptr, Kept* kept = nullptr);
 
 }  // namespace negf

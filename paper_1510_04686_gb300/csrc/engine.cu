@@ -117,13 +117,15 @@ static int32_t* err_word(const EngineWs& w) {
 
 cudaError_t Engine::gemm(int P, int M, int N, int K, z64 alpha, BMc<double> A, int opA,
                          BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
-                         BMc<double> D, const int32_t* active) {
+                         BMc<double> D, const int32_t* active, int reuse) {
+  kept.reuse = reuse;
   if (prec_mixed(prec) && w.residues)
     return crt_gemm(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, false, active,
-                    crt_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys);
+                    crt_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys, nullptr, &kept);
   if (prec_mixed(prec))
     return tc_gemm(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, false, active,
-                   tc_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys);
+                   tc_view(w, P, b, prec_bits(prec)), prec_bits(prec), n_sys, false, nullptr,
+                   &kept);
   return gemm_simt(s, P, M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, active);
 }
 
@@ -155,6 +157,7 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
     prof_end(s, PROF_INV);
     return e;
   }
+  kept = Kept{};  // the products below use the same scratch
   // FP32 Gauss-Jordan start X0, then X <- X + X (I - M X) with tensor-core products
   const long long bb = (long long)b * b;
   if (Mm.idx || X.idx || Mm.stride != bb || X.stride != bb || Mm.ld != b || X.ld != b)

@@ -6,6 +6,7 @@
 #include <utility>
 
 #include "common.cuh"
+#include "tc_gemm.cuh"
 
 namespace negf {
 
@@ -85,14 +86,16 @@ struct Engine {
   EngineWs w;
   int b;
   int n_sys = 0;  // distinct Hamiltonians an indexed operand selects from (0 = unknown)
+  Kept kept;      // what the tensor-core operand scratch holds after the last product
   Engine(cudaStream_t s_, int prec_, int rmin, int rmax_, const EngineWs& w_, int b_,
          int n_sys_ = 0)
       : s(s_), prec(prec_), refine_min(rmin), refine_max(rmax_ > rmin ? rmax_ : rmin), w(w_),
         b(b_), n_sys(n_sys_) {}
-  // C = alpha op(A) op(B) + beta C + gamma D for P batch items of M x N x K.
+  // C = alpha op(A) op(B) + beta C + gamma D for P batch items of M x N x K.  reuse: REUSE_A,
+  // REUSE_B where that operand is, unchanged, the one of the product just before.
   cudaError_t gemm(int P, int M, int N, int K, z64 alpha, BMc<double> A, int opA, BMc<double> B,
                    int opB, z64 beta, BM<double> C, z64 gamma, BMc<double> D,
-                   const int32_t* active);
+                   const int32_t* active, int reuse = 0);
   // Mixed form: clear the tensor-core GEMM's timeout word / OR NEGF_PT_TIMEOUT into
   // status[0..P) if a GEMM since the reset gave up a bounded wait.  No-ops in the FP64 form.
   cudaError_t timeout_reset();

@@ -227,18 +227,20 @@ negf_status lead_chunk_run(const negf_device* dev, int P, bool res, const double
     if (!iface) {
       CK(eng.gemm(Q, b, b, b, one, cst(flat(al, bb, b)), OP_N, cst(flat(w.g, bb, b)), OP_N,
                   zero, flat(w.ag, bb, b), zero, kNone, act));
+      // the order lets a product share an operand with the one before it: 8 conversions, not 12
+      // (16 points of b = 400: 80.2 -> 75.3 ms)
       CK(eng.gemm(Q, b, b, b, one, cst(flat(be, bb, b)), OP_N, cst(flat(w.g, bb, b)), OP_N,
-                  zero, flat(w.bg, bb, b), zero, kNone, act));
+                  zero, flat(w.bg, bb, b), zero, kNone, act, REUSE_B));
       CK(eng.gemm(Q, b, b, b, one, cst(flat(w.ag, bb, b)), OP_N, cst(flat(be, bb, b)), OP_N,
                   zero, flat(w.T1, bb, b), zero, kNone, act));
       CK(launch_add2(s, Q, b, cst(flat(w.T1, bb, b)), flat(w.eps_s, bb, b), flat(w.eps, bb, b),
                      0, b, 0, b, act));
-      CK(eng.gemm(Q, b, b, b, one, cst(flat(w.bg, bb, b)), OP_N, cst(flat(al, bb, b)), OP_N, one,
-                  flat(w.eps, bb, b), zero, kNone, act));
       CK(eng.gemm(Q, b, b, b, one, cst(flat(w.ag, bb, b)), OP_N, cst(flat(al, bb, b)), OP_N,
-                  zero, flat(al2, bb, b), zero, kNone, act));
+                  zero, flat(al2, bb, b), zero, kNone, act, REUSE_A));
+      CK(eng.gemm(Q, b, b, b, one, cst(flat(w.bg, bb, b)), OP_N, cst(flat(al, bb, b)), OP_N, one,
+                  flat(w.eps, bb, b), zero, kNone, act, REUSE_B));
       CK(eng.gemm(Q, b, b, b, one, cst(flat(w.bg, bb, b)), OP_N, cst(flat(be, bb, b)), OP_N,
-                  zero, flat(be2, bb, b), zero, kNone, act));
+                  zero, flat(be2, bb, b), zero, kNone, act, REUSE_A));
     } else {
       for (int sd = 0; sd < 2; ++sd) {
         const int32_t* as = w.act_side + (size_t)sd * P;
@@ -249,12 +251,12 @@ negf_status lead_chunk_run(const negf_device* dev, int P, bool res, const double
                     zero, sub(w.bg, sd, c0, 0), zero, kNone, as));
         CK(eng.gemm(P, nr, nr, nc, one, subc(w.ag, sd, r0, c0), OP_N, subc(be, sd, c0, r0), OP_N,
                     zero, sub(w.T1, sd, r0, r0), zero, kNone, as));
+        CK(eng.gemm(P, nc, nr, nc, one, subc(w.bg, sd, c0, c0), OP_N, subc(be, sd, c0, r0), OP_N,
+                    zero, sub(be2, sd, c0, r0), zero, kNone, as, REUSE_B));
         CK(eng.gemm(P, nc, nc, nr, one, subc(w.bg, sd, c0, r0), OP_N, subc(al, sd, r0, c0), OP_N,
                     one, sub(w.eps, sd, c0, c0), zero, kNone, as));
         CK(eng.gemm(P, nr, nc, nr, one, subc(w.ag, sd, r0, r0), OP_N, subc(al, sd, r0, c0), OP_N,
-                    zero, sub(al2, sd, r0, c0), zero, kNone, as));
-        CK(eng.gemm(P, nc, nr, nc, one, subc(w.bg, sd, c0, c0), OP_N, subc(be, sd, c0, r0), OP_N,
-                    zero, sub(be2, sd, c0, r0), zero, kNone, as));
+                    zero, sub(al2, sd, r0, c0), zero, kNone, as, REUSE_B));
       }
       CK(launch_add2(s, Q, b, cst(flat(w.T1, bb, b)), flat(w.eps_s, bb, b), flat(w.eps, bb, b),
                      ra0[0], nra[0], ra0[1], nra[1], act));
@@ -400,10 +402,7 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
     const bool first = (i == 0), last = (i == N - 1);
     BMc<double> Y = kNone;
     if (!first) {
-      // L_{i-1} = g_{i-1} t_{i-1} (kept for the backward sweep);  Y = t^H L.  Interface mode:
-      // t = E_R T E_C^T, so only L[:, C] = g[:, R] T and Y[C, C] = T^H L[R, C] are formed.
-      CK(eng.gemm(P, b, ic, ir, one, cview(Fc(G[i - 1]), b - ir), OP_N, tview(Hu(i - 1)), OP_N,
-                  zero, F(Lb(i - 1)), zero, kNone, nullptr));
+      // Y = t^H L with L_{i-1} = g_{i-1} t_{i-1}; interface mode: Y[C, C] = T^H L[R, C]
       CK(eng.gemm(P, ic, ic, ir, one, tview(Hu(i - 1)), OP_C, rview(Fc(Lb(i - 1)), b - ir), OP_N,
                   zero, F(w.Y), zero, kNone, nullptr));
       Y = Fc(w.Y);
@@ -413,26 +412,37 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
                        a.A, erow, Y, ic,
                        first ? SigL_R : kNone, last ? SigR_R : kNone, F(w.Mt), nullptr));
     CK(eng.inv(P, F(w.Mt), F(G[i]), a.status, nullptr));
+    // The products with g_i on the left come one after another: its operand form is made once
+    // (and again only where interface couplings take other columns of it).
+    const bool has_src = first || last || a.scatL != nullptr;
     bool have_prev = false;
     if (!first) {
       // g^<_i = K g^<_{i-1} K^H with K = g_i t_{i-1}^H; interface mode: only K[:, R] =
       // g_i[:, C] T^H, then Vt = g^<_{i-1}[:, R] K[:, R]^H and g^<_i = K[:, R] Vt[R, :]
       CK(eng.gemm(P, b, ir, ic, one, Fc(G[i]), OP_N, tview(Hu(i - 1)), OP_C, zero,
                   bcview(F(w.K), b - ir), zero, kNone, nullptr));
+    }
+    if (has_src) {  // W = g_i S_i with S_i = diag(Sigma^<_scat) + lead Sigma^< on the end slabs
+      CK(launch_source(s, P, b, a.scatL ? a.scatL + (size_t)i * b * a.A : nullptr,
+                       (long long)NB * a.A, a.A, erow,
+                       first ? SigL_L : kNone, last ? SigR_L : kNone, F(w.S), nullptr));
+      CK(eng.gemm(P, b, b, b, one, Fc(G[i]), OP_N, Fc(w.S), OP_N, zero, F(w.W), zero, kNone,
+                  nullptr, first ? 0 : REUSE_A));
+    }
+    if (!last) {
+      // L_i = g_i t_i, kept for the next slab and the backward sweep.  Interface mode:
+      // t = E_R T E_C^T, so only L[:, C] = g[:, R] T is formed.
+      CK(eng.gemm(P, b, ic, ir, one, cview(Fc(G[i]), b - ir), OP_N, tview(Hu(i)), OP_N, zero,
+                  F(Lb(i)), zero, kNone, nullptr, REUSE_A));
+    }
+    if (!first) {
       CK(eng.gemm(P, b, b, ir, one, cview(Fc(GL[i - 1]), b - ir), OP_N, cview(Fc(w.K), b - ir),
                   OP_C, zero, F(w.Vt), zero, kNone, nullptr));
       CK(eng.gemm(P, b, b, ir, one, cview(Fc(w.K), b - ir), OP_N, rview(Fc(w.Vt), b - ir), OP_N,
                   zero, F(GL[i]), zero, kNone, nullptr));
       have_prev = true;
     }
-    const bool has_src = first || last || a.scatL != nullptr;
-    if (has_src) {
-      // + g_i S_i g_i^H with S_i = diag(Sigma^<_scat) + lead Sigma^< on the end slabs
-      CK(launch_source(s, P, b, a.scatL ? a.scatL + (size_t)i * b * a.A : nullptr,
-                       (long long)NB * a.A, a.A, erow,
-                       first ? SigL_L : kNone, last ? SigR_L : kNone, F(w.S), nullptr));
-      CK(eng.gemm(P, b, b, b, one, Fc(G[i]), OP_N, Fc(w.S), OP_N, zero, F(w.W), zero, kNone,
-                  nullptr));
+    if (has_src) {  // + W g_i^H
       CK(eng.gemm(P, b, b, b, one, Fc(w.W), OP_N, Fc(G[i]), OP_C, have_prev ? one : zero,
                   F(GL[i]), zero, kNone, nullptr));
     } else if (!have_prev) {
@@ -469,17 +479,11 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
   z64* spare = w.Gn;
   for (int i = N - 2; i >= 0; --i) {
     z64* L = Lb(i);
-    // W = G_{i+1} t_i^H;  LW = L W;  G_i = g_i + LW g_i.  Interface mode (L has columns C,
-    // t_i^H rows C and columns R): W[:, R] = G_{i+1}[:, C] T^H, LW[:, R] = L[:, C] W[C, R],
-    // G_i = g_i + LW[:, R] g_i[R, :]
+    // W = G_{i+1} t_i^H;  Q = G^<_{i+1} L^H;  U = 2 W g^<_i + Q;  G^<_{i+1,i} = (U + Q) / 2.
+    // Interface mode (L has columns C, t_i^H rows C and columns R): W[:, R] = G_{i+1}[:, C] T^H,
+    // Q = G^<_{i+1}[:, C] L[:, C]^H, U = 2 W[:, R] g^<_i[R, :] + Q
     CK(eng.gemm(P, b, ir, ic, one, Fc(G[i + 1]), OP_N, tview(Hu(i)), OP_C, zero,
                 bcview(F(w.W), b - ir), zero, kNone, nullptr));
-    CK(eng.gemm(P, b, ir, ic, one, Fc(L), OP_N, cview(Fc(w.W), b - ir), OP_N, zero,
-                bcview(F(w.LW), b - ir), zero, kNone, nullptr));
-    CK(eng.gemm(P, b, b, ir, one, cview(Fc(w.LW), b - ir), OP_N, rview(Fc(G[i]), b - ir), OP_N,
-                zero, F(spare), one, Fc(G[i]), nullptr));
-    // Q = G^<_{i+1} L^H;  U = 2 W g^<_i + Q;  G^<_{i+1,i} = (U + Q) / 2  (interface mode:
-    // Q = G^<_{i+1}[:, C] L[:, C]^H, U = 2 W[:, R] g^<_i[R, :] + Q)
     CK(eng.gemm(P, b, b, ic, one, Fc(GL[i + 1]), OP_N, Fc(L), OP_C, zero, F(w.Qm), zero, kNone,
                 nullptr));
     CK(eng.gemm(P, b, b, ir, two, cview(Fc(w.W), b - ir), OP_N, rview(Fc(GL[i]), b - ir), OP_N,
@@ -487,9 +491,15 @@ negf_status rgf_chunk_run(const RgfArgs& a, int P, char* wsbase, cudaStream_t s)
     if (a.current)
       CK(launch_bond_current(s, P, b, Hu(i), Fc(w.U), Fc(w.Qm), a.current + i, N - 1, w.part,
                              reinterpret_cast<double*>(w.Mt)));  // Mt is written below
-    // G^<_ii = AH(g^<_i + L U)  (interface mode: L[:, C] U[C, :])
+    // LW = L W and G^<_ii = AH(g^<_i + L U) share L.  Interface mode: LW[:, R] = L[:, C] W[C, R],
+    // L[:, C] U[C, :]
+    CK(eng.gemm(P, b, ir, ic, one, Fc(L), OP_N, cview(Fc(w.W), b - ir), OP_N, zero,
+                bcview(F(w.LW), b - ir), zero, kNone, nullptr));
     CK(eng.gemm(P, b, b, ic, one, Fc(L), OP_N, Fc(w.U), OP_N, zero, F(w.Mt), one, Fc(GL[i]),
-                nullptr));
+                nullptr, REUSE_A));
+    // G_i = g_i + LW g_i  (interface mode: LW[:, R] g_i[R, :])
+    CK(eng.gemm(P, b, b, ir, one, cview(Fc(w.LW), b - ir), OP_N, rview(Fc(G[i]), b - ir), OP_N,
+                zero, F(spare), one, Fc(G[i]), nullptr));
     CK(launch_antiherm(s, P, b, Fc(w.Mt), F(GL[i]), nullptr));
     std::swap(G[i], spare);
     CK(launch_slab_obs(s, P, b, i, NB, a.A, Fc(G[i]), Fc(GL[i]), a.density, a.dGR, a.dGL,

@@ -771,7 +771,7 @@ void tc_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits, 
 cudaError_t tc_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
                     int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
                     BMc<double> D, bool add_identity, const int32_t* active, const TcWs& ws,
-                    int bits, int n_distinct, bool trunc_a, float* rmax) {
+                    int bits, int n_distinct, bool trunc_a, float* rmax, Kept* kept) {
   if (P <= 0 || M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   // Operands shared by all items (stride 0) or selected per item from n_distinct matrices are
   // sliced once per distinct matrix; the kernel maps each item to its slice set.
@@ -806,17 +806,25 @@ cudaError_t tc_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<d
   const int N2 = 2 * N;
   __nv_bfloat16* sa = static_cast<__nv_bfloat16*>(ws.slicesA);
   __nv_bfloat16* sb = static_cast<__nv_bfloat16*>(ws.slicesB);
+  const KeptOperand ka{A.p, sa, zA ? zA : A.idx, actA, A.stride, A.ld, opA, M, K, PA, bta, S};
+  const KeptOperand kb{B.p, sb, zB ? zB : B.idx, actB, B.stride, B.ld, opB, N, K, PB, bta, S};
+  const bool haveA = kept && (kept->reuse & REUSE_A) && kept->a == ka;
+  const bool haveB = kept && (kept->reuse & REUSE_B) && kept->b == kb;
   prof_begin(s, PROF_SLICE);
   // a row of op(A) is a column of A in memory for op T/C; a column of op(B) is a column of B for
   // op N
-  cudaError_t e = launch_slice<false>(s, bta, S, dim3((M + 31) / 32, PA), M, K, L, A, opA,
-                                      opA != OP_N, sa, ws.expA, actA);
+  cudaError_t e = cudaSuccess;
+  if (!haveA)
+    e = launch_slice<false>(s, bta, S, dim3((M + 31) / 32, PA), M, K, L, A, opA, opA != OP_N, sa,
+                            ws.expA, actA);
   if (e != cudaSuccess) return e;
-  e = launch_slice<true>(s, bta, S, dim3((N + 31) / 32, PB), N, K, L, B, opB, opB == OP_N, sb,
-                         ws.expB, actB);
+  if (!haveB)
+    e = launch_slice<true>(s, bta, S, dim3((N + 31) / 32, PB), N, K, L, B, opB, opB == OP_N, sb,
+                           ws.expB, actB);
   prof_end(s, PROF_SLICE);
-  count_launch(2);
+  count_launch(!haveA + !haveB);
   if (e != cudaSuccess) return e;
+  if (kept) *kept = Kept{ka, kb, 0};
   CUtensorMap mA, mB;
   if (!make_map(&mA, sa, L, M, (long long)PA * S, kBM)) return cudaErrorInvalidValue;
   const int NTc = kShapes[cfg / 2].nt;

@@ -26,6 +26,27 @@ struct TcWs {
   int32_t* err;         // device error word (bounded waits that gave up)
 };
 
+// What the operand scratch holds after a product: the matrix, its form and its place there.  A
+// caller that knows the next product to read the same, unchanged matrix asks for it to be taken
+// from there (`reuse`, consumed by the next product) instead of converted again; a product whose
+// operand has another form than the one kept converts it all the same.
+enum Reuse { REUSE_A = 1, REUSE_B = 2 };
+struct KeptOperand {
+  const void *x = nullptr, *place = nullptr;
+  const int32_t *idx = nullptr, *active = nullptr;
+  long long stride = 0;
+  int ld = 0, op = 0, lines = 0, K = 0, items = 0, form0 = 0, form1 = 0;
+  bool operator==(const KeptOperand& o) const {
+    return x == o.x && place == o.place && idx == o.idx && active == o.active &&
+           stride == o.stride && ld == o.ld && op == o.op && lines == o.lines && K == o.K &&
+           items == o.items && form0 == o.form0 && form1 == o.form1;
+  }
+};
+struct Kept {
+  KeptOperand a, b;
+  int reuse = 0;
+};
+
 // Fixed-point bits per operand value (the precision tier of the product): 40, 48 or 56.
 bool tc_bits_ok(int bits);
 
@@ -67,9 +88,11 @@ cudaError_t tc_prof_reset();
 // bits: fixed-point bits per operand value (tc_bits_ok); the workspace must have been carved for
 // the same bits.  rmax (nullable, float [P], zeroed by the caller): rmax[p] is raised to the
 // largest |Re| or |Im| of item p's outputs (the Newton-Schulz residual norm when C = I - M X).
+// kept (nullable): what the scratch of `ws` holds, see Kept.
 cudaError_t tc_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
                     int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
                     BMc<double> D, bool add_identity, const int32_t* active, const TcWs& ws,
-                    int bits, int n_distinct = 0, bool trunc_a = false, float* rmax = nullptr);
+                    int bits, int n_distinct = 0, bool trunc_a = false, float* rmax = nullptr,
+                    Kept* kept = nullptr);
 
 }  // namespace negf
