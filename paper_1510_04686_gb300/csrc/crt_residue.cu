@@ -1,4 +1,6 @@
 // Operand residue kernels of the tensor-core complex GEMM (see crt_residue.cuh, crt_plan.cuh).
+#include <cmath>
+
 #include "f32x2.cuh"
 #include "crt_residue.cuh"
 
@@ -7,7 +9,8 @@ namespace {
 
 // ------------------------------------------------------------------ line norm
 // Sum of squares of |x| relative to 2^ex, ex the largest biased exponent so far.  The leading 20
-// mantissa bits are used (truncated; scale_of allows for it).
+// mantissa bits are used (truncated; scale_of allows for it), a subnormal value counts as the next
+// larger number with an implicit bit.
 struct Norm {
   int ex;
   float s;
@@ -15,16 +18,29 @@ struct Norm {
 __device__ __forceinline__ float pow2m(int d) {  // 2^-d, 0 <= d; 0 beyond FP32's range
   return d > 126 ? 0.0f : __int_as_float((127 - d) << 23);
 }
-__device__ __forceinline__ void norm_add(Norm& n, double x) {
-  const unsigned h = (unsigned)(__double2hiint(x)) & 0x7FFFFFFFu;
-  const int e = max((int)(h >> 20), 1);
-  if (e > n.ex) {
-    n.s *= pow2m(2 * (e - n.ex));
-    n.ex = e;
+// n complex values at once: one test for a larger exponent, and the FP32 value of each mantissa and
+// relative exponent by a shift and a subtraction of the high word.
+template <int n>
+__device__ __forceinline__ void norm_add(Norm& nm, const z64* v) {
+  int h[2 * n], top = 1 << 20;
+#pragma unroll
+  for (int i = 0; i < 2 * n; ++i) {
+    const double x = i & 1 ? v[i / 2].im : v[i / 2].re;
+    h[i] = (__double2hiint(x) & 0x7FFFFFFF) | (int)min((unsigned)__double2loint(x), 1u);
+    top = max(top, h[i]);
   }
-  const float m = __int_as_float(0x3F800000 | ((h & 0xFFFFFu) << 3));  // [1, 2)
-  const float f = (h | (unsigned)__double2loint(x)) ? m * pow2m(n.ex - e) : 0.0f;
-  n.s = fmaf(f, f, n.s);
+  top >>= 20;
+  if (top > nm.ex) {
+    nm.s *= pow2m(2 * (top - nm.ex));
+    nm.ex = top;
+  }
+  const int low = max((nm.ex - 126) << 20, 1);  // below: zero, or nothing next to 2^ex
+  const unsigned off = (unsigned)(nm.ex - 127) << 23;
+#pragma unroll
+  for (int i = 0; i < 2 * n; ++i) {
+    const float f = h[i] >= low ? __uint_as_float(((unsigned)h[i] << 3) - off) : 0.0f;
+    nm.s = fmaf(f, f, nm.s);
+  }
 }
 __device__ __forceinline__ void norm_merge(Norm& n, int oe, float os) {
   const int e = max(n.ex, oe);
@@ -36,33 +52,36 @@ __device__ __forceinline__ Norm norm_warp(Norm n) {
     norm_merge(n, __shfl_xor_sync(0xffffffffu, n.ex, o), __shfl_xor_sync(0xffffffffu, n.s, o));
   return n;
 }
-// Exponent e with 2-norm 2^e < 2^alpha for the line; kNonFinite when it holds an infinity or NaN.
-__device__ __forceinline__ int scale_of(Norm n, int alpha) {
+// Exponent e with sigma 2-norm 2^e < 2^alpha for the line; kNonFinite when it holds an infinity or
+// NaN.
+__device__ __forceinline__ int scale_of(Norm n, int alpha, float sigma2) {
   if (n.ex >= 0x7FF) return kNonFinite;
   if (!(n.s > 0.0f)) return 0;
   // truncated mantissas and the FP32 sum make s at most 2^-8 too small in relative terms
   int x;
-  frexpf(n.s * 1.00390625f, &x);  // norm < 2^(x / 2 + ex - 1023)
+  frexpf(n.s * sigma2 * 1.00390625f, &x);  // norm < 2^(x / 2 + ex - 1023)
   return alpha - ((x + 1) >> 1) - (n.ex - 1023);
 }
 
 // ------------------------------------------------------------------ residues
-// round(x 2^e) plus 128 in every digit position, so that byte i of the result is the balanced
-// digit i plus 128.  |x| 2^e < 2^61.
-__device__ __forceinline__ unsigned long long biased(double x, int e, bool flip) {
+// round(sigma x 2^e) plus 128 in every digit position, so that byte i of the result is the balanced
+// digit i plus 128.  sig = sigma 2^64 (0: sigma is one).  flip: 0x80000000 changes the sign of x.
+// The scaled line's norm is below 2^alpha, alpha <= 60, so |sigma x 2^e| is the mantissa, aligned to
+// the top of 64 bits, shifted right by three or more; 64 and beyond leave nothing.
+__device__ __forceinline__ unsigned long long biased(double x, int e, unsigned flip,
+                                                     unsigned long long sig) {
   constexpr unsigned long long kBias = 0x8080808080808080ull;
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((u >> 52) & 0x7FF);
-  unsigned long long m = u & 0xFFFFFFFFFFFFFull;
-  if (ex) m |= 1ull << 52;
-  const int sh = (ex ? ex : 1) - 1075 + e;  // |x| 2^e = m 2^sh
-  unsigned long long r;
-  if (sh >= 0)
-    r = m << min(sh, 63);
-  else
-    r = sh <= -64 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
-  const bool neg = ((u >> 63) != 0) != flip;
-  return (neg ? 0ull - r : r) + kBias;
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int ex = (int)((hi >> 20) & 0x7FF);
+  const unsigned mh = (hi & 0xFFFFFu) | (ex ? 0x100000u : 0u);
+  unsigned long long m =
+      (unsigned long long)__funnelshift_l(lo, mh, 11) << 32 | (unsigned long long)(lo << 11);
+  if (sig) m = __umul64hi(m, sig);
+  unsigned long long r;  // a shift by 64 or more gives zero
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"((unsigned)(1085 - max(ex, 1) - e)));
+  r = (r + 1) >> 1;
+  const long long neg = (long long)((int)(hi ^ flip) >> 31);  // 0 or -1
+  return (r ^ (unsigned long long)neg) + (kBias - (unsigned long long)neg);
 }
 // Digits 2 t and 2 t + 1 of a biased value as a BF16 pair; sel = the byte selector of t.  A byte b
 // is (128 + its low seven bits, exact with the exponent of 128) - (128 or 256 by its top bit).
@@ -83,14 +102,13 @@ __device__ __forceinline__ void mma_16x8x16(float* d, const uint32_t* a, uint32_
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
 }
-// Two integers below 2^24 modulo p (balanced to within one unit), as a BF16 pair.  x / p rounds to
-// the nearest integer in the single rounding of the FMA.
-__device__ __forceinline__ uint32_t residue_bf16(float x0, float x1, f2 invp, f2 negp) {
+// Two integers below 2^24 modulo p (balanced to within one unit).  x / p rounds to the nearest
+// integer in the single rounding of the FMA.
+__device__ __forceinline__ f2 residues(f2 x, f2 invp, f2 negp) {
   const f2 magic = pack2(12582912.0f, 12582912.0f), unmagic = pack2(-12582912.0f, -12582912.0f);
-  const f2 x = pack2(x0, x1);
-  const f2 r = fma2(add2(fma2(x, invp, magic), unmagic), negp, x);
-  float lo, hi;
-  unpack2(r, lo, hi);
+  return fma2(add2(fma2(x, invp, magic), unmagic), negp, x);
+}
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
   const __nv_bfloat162 w = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&w);
 }
@@ -145,8 +163,12 @@ __device__ __forceinline__ void write_planes(const ResidueConst& rc, const Coef&
       for (int b = 0; b < NB; ++b) {
         float d[4];
         mma_16x8x16(d, a, b0[b], b1[b]);
-        u[b][i] = residue_bf16(d[0], d[2], invp[b], negp[b]);
-        v[b][i] = residue_bf16(d[1], d[3], invp[b], negp[b]);
+        // neighbouring accumulators (u and v of one value) form the pairs without moves
+        float u0, v0, u1, v1;
+        unpack2(residues(pack2(d[0], d[1]), invp[b], negp[b]), u0, v0);
+        unpack2(residues(pack2(d[2], d[3]), invp[b], negp[b]), u1, v1);
+        u[b][i] = bf16_pair(u0, u1);
+        v[b][i] = bf16_pair(v0, v1);
       }
     }
     if (!in) continue;
@@ -168,12 +190,15 @@ __device__ __forceinline__ void write_planes(const ResidueConst& rc, const Coef&
 // 16 x 16 digit matrices (rows: values, columns: the digits of Re and Im) times the 16 x 2 n
 // constants, whose results are reduced modulo p in registers; a lane ends up with eight
 // neighbouring values of a residue plane and stores them as 16 bytes, 128 contiguous bytes per
-// plane and warp.  Bound by instruction issue (450 per value and 12 moduli; 2.85 us per 400 x 400
-// operand, 3.6 TB/s of reads and writes).
+// plane and warp.  Bound by instruction issue, so that what counts is instructions per value: norms
+// take the FP32 value of a mantissa by a shift and a subtraction, sigma is a 64-bit integer
+// multiplication (as an FP64 one it held the two-lane FP64 pipe for a fifth of the kernel), and u and
+// v of a value are reduced as the neighbouring accumulators that they are.  A 64 x 400^3 product with
+// both its operands: 864 -> 817 us, the two conversions about 365 -> 320.
 template <int LINES, int NB>
 __global__ void __launch_bounds__(kThreads)
-    k_residue_strip(const __grid_constant__ ResidueConst rc, int n, int alpha, double sigma,
-                    int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
+    k_residue_strip(const __grid_constant__ ResidueConst rc, int n, int alpha, unsigned long long sig,
+                    float sigma2, int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
                     __nv_bfloat16* out, int32_t* eo, const int32_t* active) {
   static_assert(kWarps % LINES == 0 && 32 % LINES == 0, "warps and lanes per line");
   const int p = blockIdx.y;
@@ -193,11 +218,10 @@ __global__ void __launch_bounds__(kThreads)
   constexpr int kPerLine = kWarps / LINES;
   const int li = line_is_col ? lane % LINES : w / kPerLine;
   const int k0 = line_is_col ? w * (32 / LINES) + lane / LINES : (w % kPerLine) * 32 + lane;
-  constexpr int kStep = kThreads / LINES, kLoads = 2;
+  constexpr int kStep = kThreads / LINES, kLoads = 4;
   const bool have = l0 + li < n_lines;
   const long long estride = line_is_col ? X.ld : 1;
   const z64* src = x + (line_is_col ? (long long)(l0 + li) : (long long)(l0 + li) * X.ld);
-  const bool scale = sigma != 1.0;
   Norm nm{1, 0.0f};
   for (int kb = k0; kb < L; kb += kLoads * kStep) {
     z64 v[kLoads];
@@ -207,12 +231,12 @@ __global__ void __launch_bounds__(kThreads)
       v[u] = have && k < K ? src[k * estride] : mkc(0.0, 0.0);
     }
 #pragma unroll
-    for (int u = 0; u < kLoads; ++u) {
+    for (int u = 0; u < kLoads; u += 2) {
       const int k = kb + u * kStep;
-      if (scale) v[u] = mkc(sigma * v[u].re, sigma * v[u].im);
-      norm_add(nm, v[u].re);
-      norm_add(nm, v[u].im);
-      if (k < L) strip[li * lds + padded(k)] = v[u];
+      if (k >= L) break;
+      norm_add<2>(nm, v + u);
+      strip[li * lds + padded(k)] = v[u];
+      if (k + kStep < L) strip[li * lds + padded(k + kStep)] = v[u + 1];
     }
   }
   if (line_is_col) {
@@ -230,20 +254,21 @@ __global__ void __launch_bounds__(kThreads)
     const int first = line_is_col ? 0 : line * kPerLine, count = line_is_col ? kWarps : kPerLine;
     Norm t = part[first][line];
     for (int i = 1; i < count; ++i) norm_merge(t, part[first + i][line].ex, part[first + i][line].s);
-    const int e = scale_of(t, alpha);
+    const int e = scale_of(t, alpha, sigma2);
     sexp[line] = e;
     if (l0 + line < n_lines)
       eo[(long long)p * n_lines + l0 + line] = e == kNonFinite ? kNonFinite : -e;
   }
   __syncthreads();
   {  // each thread converts the elements that it loaded
-    const bool conj = (op == OP_C), fine = sexp[li] != kNonFinite;
+    const bool fine = sexp[li] != kNonFinite;
+    const unsigned conj = op == OP_C ? 0x80000000u : 0u;
     const int e = fine ? sexp[li] : 0;
 #pragma unroll 2
     for (int k = k0; k < L; k += kStep) {
       const int at = li * lds + padded(k);
       const z64 v = fine ? strip[at] : mkc(0.0, 0.0);
-      ints[at] = make_ulonglong2(biased(v.re, e, false), biased(v.im, e, conj));
+      ints[at] = make_ulonglong2(biased(v.re, e, 0u, sig), biased(v.im, e, conj, sig));
     }
   }
   __syncthreads();
@@ -256,8 +281,8 @@ __global__ void __launch_bounds__(kThreads)
 constexpr int kSegment = 4096;
 template <int NB>
 __global__ void __launch_bounds__(kThreads)
-    k_residue_long(const __grid_constant__ ResidueConst rc, int n, int alpha, double sigma,
-                   int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
+    k_residue_long(const __grid_constant__ ResidueConst rc, int n, int alpha, unsigned long long sig,
+                   float sigma2, int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
                    __nv_bfloat16* out, int32_t* eo, const int32_t* active) {
   const int p = blockIdx.y;
   if (active && !active[p]) return;
@@ -273,25 +298,25 @@ __global__ void __launch_bounds__(kThreads)
   Norm nm{1, 0.0f};
   for (int k = threadIdx.x; k < K; k += kThreads) {
     const z64 v = src[k * estride];
-    norm_add(nm, sigma * v.re);
-    norm_add(nm, sigma * v.im);
+    norm_add<1>(nm, &v);
   }
   nm = norm_warp(nm);
   if (lane == 0) part[w] = nm;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < kWarps; ++i) norm_merge(nm, part[i].ex, part[i].s);
-    sexp = scale_of(nm, alpha);
+    sexp = scale_of(nm, alpha, sigma2);
     eo[(long long)p * n_lines + line] = sexp == kNonFinite ? kNonFinite : -sexp;
   }
   __syncthreads();
-  const bool conj = (op == OP_C), fine = sexp != kNonFinite;
+  const bool fine = sexp != kNonFinite;
+  const unsigned conj = op == OP_C ? 0x80000000u : 0u;
   const int e = fine ? sexp : 0;
   for (int s0 = 0; s0 < L; s0 += kSegment) {
     const int len = min(kSegment, L - s0);
     for (int k = threadIdx.x; k < len; k += kThreads) {
       const z64 v = fine && s0 + k < K ? src[(s0 + k) * estride] : mkc(0.0, 0.0);
-      ints[padded(k)] = make_ulonglong2(biased(sigma * v.re, e, false), biased(sigma * v.im, e, conj));
+      ints[padded(k)] = make_ulonglong2(biased(v.re, e, 0u, sig), biased(v.im, e, conj, sig));
     }
     __syncthreads();
     write_planes<1, NB>(rc, coef, n, ints, 0, line, n_lines, s0, len, L,
@@ -310,8 +335,8 @@ __host__ constexpr size_t strip_bytes(int lines, int L) {
 
 namespace {
 template <int LINES, int NB>
-cudaError_t launch_strip(cudaStream_t s, const CrtPlan& pl, int alpha, double sigma, int items,
-                         int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
+cudaError_t launch_strip(cudaStream_t s, const CrtPlan& pl, int alpha, unsigned long long sig,
+                         float sigma2, int items, int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
                          __nv_bfloat16* out, int32_t* eo, const int32_t* active) {
   static std::atomic<unsigned> attr{0};
   cudaError_t e = set_smem_once(attr, reinterpret_cast<const void*>(&k_residue_strip<LINES, NB>),
@@ -319,24 +344,24 @@ cudaError_t launch_strip(cudaStream_t s, const CrtPlan& pl, int alpha, double si
   if (e != cudaSuccess) return e;
   const dim3 grid((n_lines + LINES - 1) / LINES, items);
   k_residue_strip<LINES, NB><<<grid, kThreads, strip_bytes(LINES, L), s>>>(
-      residue_const(pl), pl.n, alpha, sigma, n_lines, K, L, X, op, line_is_col, out, eo, active);
+      residue_const(pl), pl.n, alpha, sig, sigma2, n_lines, K, L, X, op, line_is_col, out, eo, active);
   return cudaGetLastError();
 }
 template <int LINES>
-cudaError_t launch_strip(cudaStream_t s, const CrtPlan& pl, int alpha, double sigma, int items,
-                         int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
+cudaError_t launch_strip(cudaStream_t s, const CrtPlan& pl, int alpha, unsigned long long sig,
+                         float sigma2, int items, int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
                          __nv_bfloat16* out, int32_t* eo, const int32_t* active) {
   if (pl.n <= 12)
-    return launch_strip<LINES, 3>(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col,
+    return launch_strip<LINES, 3>(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col,
                                   out, eo, active);
-  return launch_strip<LINES, 4>(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col,
+  return launch_strip<LINES, 4>(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col,
                                 out, eo, active);
 }
 }  // namespace
 
 namespace {
-cudaError_t launch_long(cudaStream_t s, const CrtPlan& pl, int alpha, double sigma, int items,
-                        int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
+cudaError_t launch_long(cudaStream_t s, const CrtPlan& pl, int alpha, unsigned long long sig,
+                        float sigma2, int items, int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
                         __nv_bfloat16* out, int32_t* eo, const int32_t* active) {
   auto* fn = pl.n <= 12 ? &k_residue_long<3> : &k_residue_long<4>;
   static std::atomic<unsigned> attr[2];
@@ -344,7 +369,7 @@ cudaError_t launch_long(cudaStream_t s, const CrtPlan& pl, int alpha, double sig
   cudaError_t e = set_smem_once(attr[pl.n <= 12 ? 0 : 1], reinterpret_cast<const void*>(fn),
                                 (int)smem);
   if (e != cudaSuccess) return e;
-  fn<<<dim3(n_lines, items), kThreads, smem, s>>>(residue_const(pl), pl.n, alpha, sigma, n_lines, K,
+  fn<<<dim3(n_lines, items), kThreads, smem, s>>>(residue_const(pl), pl.n, alpha, sig, sigma2, n_lines, K,
                                                   L, X, op, line_is_col, out, eo, active);
   return cudaGetLastError();
 }
@@ -353,22 +378,24 @@ cudaError_t launch_long(cudaStream_t s, const CrtPlan& pl, int alpha, double sig
 cudaError_t launch_residues(cudaStream_t s, const CrtPlan& pl, int alpha, double sigma, int items,
                             int n_lines, int K, int L, BMc<double> X, int op, bool line_is_col,
                             __nv_bfloat16* out, int32_t* eo, const int32_t* active) {
+  const unsigned long long sig = sigma < 1.0 ? (unsigned long long)ldexp(sigma, 64) : 0ull;
+  const float sigma2 = (float)(sigma * sigma);
   // eight lines per CTA while three CTAs fit an SM (the constants and the reductions are then a
   // small part of a CTA's work), fewer for longer lines
   constexpr size_t kThree = 74 * 1024;
   if (strip_bytes(8, L) <= kThree)
-    return launch_strip<8>(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col, out, eo,
+    return launch_strip<8>(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col, out, eo,
                            active);
   if (strip_bytes(4, L) <= kThree)
-    return launch_strip<4>(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col, out, eo,
+    return launch_strip<4>(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col, out, eo,
                            active);
   if (strip_bytes(2, L) <= kThree)
-    return launch_strip<2>(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col, out, eo,
+    return launch_strip<2>(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col, out, eo,
                            active);
   if (strip_bytes(1, L) <= kStripBytes)
-    return launch_strip<1>(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col, out, eo,
+    return launch_strip<1>(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col, out, eo,
                            active);
-  return launch_long(s, pl, alpha, sigma, items, n_lines, K, L, X, op, line_is_col, out, eo,
+  return launch_long(s, pl, alpha, sig, sigma2, items, n_lines, K, L, X, op, line_is_col, out, eo,
                      active);
 }
 
