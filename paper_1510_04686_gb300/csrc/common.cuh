@@ -98,6 +98,30 @@ __device__ __forceinline__ cx<R>* bat(BM<R> a, int p) {
   return a.p + (a.idx ? (long long)a.idx[p] : (long long)p) * a.stride;
 }
 
+// Chains of short kernels: a kernel launched by launch_chained may be set up while the one before it
+// on the stream still runs (once all of that one's CTAs have started and called chain_next), and
+// waits in chain_wait, first thing, until it has finished with its writes visible.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // ---- launchers (all asynchronous on `s`) ----------------------------------------------
 
 // C[p] = alpha op(A[p]) op(B[p]) + beta C[p] + gamma D[p] on the CUDA cores (FP64 form).

@@ -113,6 +113,8 @@ constexpr int kStripRows = 4, kStripCols = 8, kStripWarps = 4, kStripAhead = 4;
 __global__ void __launch_bounds__(32 * kStripWarps)
     k_gemm_strip(int M, int N, int K, z64 alpha, BMc<double> A, int opA, BMc<double> B, int opB,
                  z64 beta, BM<double> C, z64 gamma, BMc<double> D, const int32_t* active) {
+  chain_next();
+  chain_wait();
   const int p = blockIdx.y;
   if (active && !active[p]) return;
   const int lane = threadIdx.x & 31;
@@ -185,12 +187,12 @@ cudaError_t gemm_simt(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc
     // CTAs per item: enough to fill the chip, few enough that masked items cost little
     const long long most = std::max(64ll, 152ll * 8 / P);
     const unsigned ctas = (unsigned)std::min(most, (strips + kStripWarps - 1) / kStripWarps);
-    k_gemm_strip<<<dim3(ctas, P), 32 * kStripWarps, 0, s>>>(M, N, K, alpha, A, opA, B, opB, beta,
-                                                           C, gamma, D, active);
-  } else {
-    const dim3 grid((N + BNT - 1) / BNT, (M + BMT - 1) / BMT, P);
-    k_gemm_simt<<<grid, 256, 0, s>>>(M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, active);
+    count_launch();
+    return launch_chained(&k_gemm_strip, dim3(ctas, P), dim3(32 * kStripWarps), 0, s, M, N, K,
+                          alpha, A, opA, B, opB, beta, C, gamma, D, active);
   }
+  const dim3 grid((N + BNT - 1) / BNT, (M + BMT - 1) / BMT, P);
+  k_gemm_simt<<<grid, 256, 0, s>>>(M, N, K, alpha, A, opA, B, opB, beta, C, gamma, D, active);
   count_launch();
   return cudaGetLastError();
 }
