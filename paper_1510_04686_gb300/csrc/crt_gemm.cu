@@ -109,11 +109,16 @@ __device__ __forceinline__ bool pairs_aligned(const void* p, long long stride, i
 // instead of eight keep the integer multiply-adds of the reconstruction (the busiest pipe of the
 // epilogue) behind the MMAs; one elected lane issues TMA and MMA (elect.sync instead of a test of
 // the lane number took the MMA issue from 479 to 360 us per 76 items).
-template <int NT>
+template <int NT, bool HP>
 struct Cfg {
   static constexpr int kABox = kBM * kKC * 2;
   static constexpr int kBBox = NT * kKC * 2;
-  static constexpr int kStage = kABox + kBBox;
+  static constexpr int kChunk = kABox + kBBox;
+  // K chunks per stage.  Narrow tiles have little to do between a stage's barriers: two chunks per
+  // stage take 37 items of 333 x 217 x 591 from 490 to 473 us.  Wide ones need the stages: 64 items
+  // of 400^3 823 -> 850 us; nor do the correction sums leave the issuer waiting (603 -> 616 us).
+  static constexpr int kPer = NT <= 64 && !HP ? 2 : 1;
+  static constexpr int kStage = kPer * kChunk;
   static constexpr int kStages = std::min(10, (227 * 1024 - 1280) / kStage);
   static_assert(kBBox % 1024 == 0, "stages keep the 1024-byte alignment of the swizzle");
   static constexpr int kSmem = kStages * kStage + 1024 + 256;  // + align + barriers
@@ -139,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const int32_t* __restrict__ zidxB, int zmodeB, z64 alpha, z64 beta, z64 gamma,
               BM<double> C, BMc<double> D, int add_identity, const int32_t* active, int32_t* err,
               float* rmax, int count_flops) {
-  using CF = Cfg<NT>;
+  using CF = Cfg<NT, HP>;
   constexpr int kStages = CF::kStages;
   constexpr int kCols = NT / 4;            // columns per epilogue warp
   constexpr int kFin = 4;                  // columns per round of the final pass
@@ -204,15 +209,21 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int step = h >> 1, mod = step / parts, part = step - mod * parts;
           const int z = 2 * mod + (h & 1);
           const int lo = part * part_k16, hi = min(k16, lo + part_k16);
-          for (int kc = lo; kc < hi; kc += kKC / 16) {
+          for (int kc = lo; kc < hi; kc += CF::kPer * kKC / 16) {
             if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) {
               ok = false;
               break;
             }
             unsigned char* st = smem + stage * CF::kStage;
-            mbar_expect_tx(&full[stage], bytes);
+            const bool two = CF::kPer == 2 && hi - kc > kKC / 16;
+            mbar_expect_tx(&full[stage], two ? 2 * bytes : bytes);
             tma_load_3d(st, &mapA, &full[stage], kc * 16, m0, zA + z);
             tma_load_3d(st + CF::kABox, &mapB, &full[stage], kc * 16, n0, zB + z);
+            if (two) {
+              st += CF::kChunk;
+              tma_load_3d(st, &mapA, &full[stage], kc * 16 + kKC, m0, zA + z);
+              tma_load_3d(st + CF::kABox, &mapB, &full[stage], kc * 16 + kKC, n0, zB + z);
+            }
             if (++stage == kStages) {
               stage = 0;
               phase ^= 1;
@@ -251,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int part = (h >> 1) % parts;
           const int lo = part * part_k16, hi = min(k16, lo + part_k16);
           uint32_t acc_on = 0;
-          for (int kc = lo; kc < hi; kc += kKC / 16) {
+          for (int kc = lo; kc < hi; kc += CF::kPer * kKC / 16) {
             if (!mbar_wait(&full[stage], phase, abort_flag)) {
               ok = false;
               break;
@@ -261,9 +272,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t da = sw128_desc(a), db = sw128_desc(b);
             const int nk = hi - kc;  // K steps left in this part
 #pragma unroll
-            for (int k = 0; k < kKC / 16; ++k) {
-              if (k < nk)  // one K step is 32 bytes along the swizzled row
-                mma_bf16(dcol, da + 2 * k, db + 2 * k, idesc, k == 0 ? acc_on : 1u);
+            for (int k = 0; k < CF::kPer * kKC / 16; ++k) {
+              // one K step is 32 bytes along the swizzled row of its chunk
+              constexpr int kPerChunk = kKC / 16;
+              const uint64_t at = k / kPerChunk * (CF::kChunk >> 4) + k % kPerChunk * 2;
+              if (k < nk) mma_bf16(dcol, da + at, db + at, idesc, k == 0 ? acc_on : 1u);
             }
             acc_on = 1;
             mma_commit(&empty[stage]);
@@ -567,7 +580,7 @@ int sm_count() {
 
 template <int NT, bool HP>
 cudaError_t launch_crt(cudaStream_t s, const GemmArgs& a) {
-  using CF = Cfg<NT>;
+  using CF = Cfg<NT, HP>;
   static std::atomic<unsigned> attr{0};
   cudaError_t e =
       set_smem_once(attr, reinterpret_cast<const void*>(&k_crt_gemm<NT, HP>), CF::kSmem);
