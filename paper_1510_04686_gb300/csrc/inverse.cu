@@ -621,6 +621,67 @@ __global__ void __launch_bounds__(256) k_gj_update32(int n, int k0, int w, int n
     }
 }
 
+// The same update for panels of at most four columns (blocks beyond 2425), which memory bounds: one
+// read and one write of the matrix for four complex multiply-adds per element.  No tile is worth
+// staging there; a thread keeps its 2 x 8 elements (rows of a warp, columns 32 apart) and the pivot
+// rows of its columns in registers, so that 16 loads per thread are under way.  The sums are those of
+// k_gj_update32, in its order.  n = 3430: two slabs solved in 345 ms with the tiles, 325 with this kernel (the tiles
+// took 48 us per update, 3.9 TB/s); at n = 2400, eight columns, the tiles are faster (31.6 ms against
+// 32.3 for an inverse).
+constexpr int kThinPanel = 4, kThinRows = 8, kThinCols = 64, kThinWarps = 8;
+__global__ void __launch_bounds__(32 * kThinWarps)
+    k_gj_update_thin(int n, int k0, int w, int nb, const cx<float>* U, const cx<float>* srcs,
+                     cx<float>* dsts, const int32_t* conts, const int32_t* active) {
+  chain_next();
+  chain_wait();
+  const int p = blockIdx.z;
+  if (active && !active[p]) return;
+  __shared__ cx<float> Us[kThinWarps * kThinRows][kThinPanel];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int m0 = blockIdx.y * kThinWarps * kThinRows, n0 = blockIdx.x * kThinCols + lane;
+  const long long nn = (long long)n * n;
+  const cx<float>* u = U + (long long)p * n * nb;
+  const cx<float>* src = srcs + p * nn;
+  cx<float>* dst = dsts + p * nn;
+  const int32_t* cont = conts + (long long)p * n;
+  const cx<float> zero = mkc<float>(0.0f, 0.0f);
+  cx<float> acc[kThinRows][2], t[kThinPanel][2];
+#pragma unroll
+  for (int i = 0; i < kThinRows; ++i) {
+    const int r = m0 + wid * kThinRows + i;
+    const bool keep = r < n && (r < k0 || r >= k0 + w);
+    const cx<float>* row = src + (long long)(keep ? cont[r] : 0) * n;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) acc[i][j] = keep && n0 + 32 * j < n ? row[n0 + 32 * j] : zero;
+  }
+#pragma unroll
+  for (int k = 0; k < kThinPanel; ++k) {
+    const cx<float>* row = src + (long long)(k < w ? cont[k0 + k] : 0) * n;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) t[k][j] = k < w && n0 + 32 * j < n ? row[n0 + 32 * j] : zero;
+  }
+  for (int e = threadIdx.x; e < kThinWarps * kThinRows * kThinPanel; e += 32 * kThinWarps) {
+    const int r = m0 + e / kThinPanel, k = e % kThinPanel;
+    Us[e / kThinPanel][k] = r < n && k < w ? u[(long long)r * nb + k] : zero;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kThinPanel; ++k) {
+    if (k >= w) break;
+#pragma unroll
+    for (int i = 0; i < kThinRows; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) cfma(acc[i][j], Us[wid * kThinRows + i][k], t[k][j]);
+  }
+#pragma unroll
+  for (int i = 0; i < kThinRows; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int r = m0 + wid * kThinRows + i, col = n0 + 32 * j;
+      if (r < n && col < n && (col < k0 || col >= k0 + w)) dst[(long long)r * n + col] = acc[i][j];
+    }
+}
+
 // Column permutation that the pivoting left: column c of the inverse is column map[c] of the
 // eliminated matrix.  A chain of exchanges, so one thread per item follows it in shared memory.
 __global__ void __launch_bounds__(kThreads) k_gj_perm(int n, const int32_t* piv, int32_t* map,
@@ -835,8 +896,15 @@ cudaError_t gj_inverse32(cudaStream_t s, int P, int n, BM<double> M, BM<double> 
     e = panel32(s, P, n, k0, w, nb, src, dst, U, piv, map, status, active);
     prof_end(s, PROF_GJ_PANEL);
     if (e != cudaSuccess) return e;
-    e = launch_chained(&k_gj_update32, grid, dim3(256), 0, s, n, k0, w, nb, U, src, dst, map,
-                       active);
+    if (nb <= kThinPanel) {
+      constexpr int kRows = kThinWarps * kThinRows;
+      const dim3 thin((n + kThinCols - 1) / kThinCols, (n + kRows - 1) / kRows, P);
+      e = launch_chained(&k_gj_update_thin, thin, dim3(32 * kThinWarps), 0, s, n, k0, w, nb, U,
+                         src, dst, map, active);
+    } else {
+      e = launch_chained(&k_gj_update32, grid, dim3(256), 0, s, n, k0, w, nb, U, src, dst, map,
+                         active);
+    }
     count_launch();
     if (e != cudaSuccess) return e;
     std::swap(src, dst);
