@@ -249,6 +249,147 @@ __global__ void __launch_bounds__(kThreads) k_gj_small(int n, BM<R> Mm, BM<R> X,
       x[(long long)r * X.ld + c] = A[r * n + src[c]];
 }
 
+// The multiply-adds of a step are written out, each rounding in its place, so that the result does
+// not depend on how the compiler contracts them.  `other` takes the imaginary part's products in
+// the other order: the elimination has always done so in the rows that its unrolling by four left
+// over, and the results stay the same bit for bit.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+template <typename R>
+__device__ __forceinline__ cx<R> cmul(cx<R> a, cx<R> b) {
+  return mkc<R>(fma_rn(a.re, b.re, -mul_rn(a.im, b.im)), fma_rn(a.re, b.im, mul_rn(a.im, b.re)));
+}
+template <typename R>
+__device__ __forceinline__ void eliminate(cx<R>& x, cx<R> f, cx<R> p, bool other) {
+  x.re = sub_rn(x.re, fma_rn(f.re, p.re, -mul_rn(f.im, p.im)));
+  // (a product has the same rounding whichever factor comes first)
+  const R a = other ? f.re : f.im, b = other ? p.im : p.re;
+  const R c = other ? f.im : f.re, d = other ? p.re : p.im;
+  x.im = sub_rn(x.im, fma_rn(a, b, mul_rn(c, d)));
+}
+
+// One CTA per matrix, the whole matrix in shared memory.  A step's chain (largest entry of the
+// column, reciprocal) is as long as its update: FP64 issues two lanes per clock and SM, and a
+// division is some twenty operations one after another.  So the first warp updates the next column
+// ahead of the rest and finds that column's pivot and reciprocal while the other warps update the
+// remaining columns.  128 blocks of 40: 284 -> 230 us, 16 of 64: 682 -> 588, 30 of 106: 2436 -> 2225.
+// (Padded rows and a scheduler kept free for the chain gave nothing more.  FP32 has no such pipe: there
+// the single warp's column is what a step waits for, 8 blocks of 100 680 -> 946 us, so it keeps the
+// form above.)
+__global__ void __launch_bounds__(kThreads) k_gj_small64(int n, BM<double> Mm, BM<double> X,
+                                                         int32_t* status, const int32_t* active) {
+  const int p = blockIdx.x;
+  if (active && !active[p]) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  z64* A = reinterpret_cast<z64*>(smem_raw);
+  z64* f = A + (size_t)n * n;  // the pivot column
+  z64* prow = f + n;            // the scaled pivot row
+  int* perm = reinterpret_cast<int*>(prow + n);
+  int* src = perm + n;
+  __shared__ unsigned char other[kThreads];  // n <= kThreads (gj_fits_small)
+  __shared__ z64 recip;
+  __shared__ int pivot;
+  int32_t* st = status ? status + p : nullptr;
+  const z64* m = bat(Mm, p);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const z64 zero = mkc(0.0, 0.0);
+  for (int r = 0; r < n; ++r)
+    for (int c = tid; c < n; c += kThreads) A[r * n + c] = m[(long long)r * Mm.ld + c];
+  const int old = kThreads / n;  // rows per step of the elimination unrolled by four
+  if (tid < n) other[tid] = tid % old + (tid / (4 * old) * 4 + 3) * old >= n;
+  __syncthreads();
+  // the pivot of column j among rows [j, n) and its reciprocal (first warp)
+  auto search = [&](int j) {
+    Mag<double> best{-1.0, 0.0};
+    int bi = n;
+    for (int r = lane; r < n; r += 32) {
+      if (r < j) continue;
+      const Mag<double> v = mag2(A[r * n + j]);
+      if (better(v, r, best, bi)) {
+        best = v;
+        bi = r;
+      }
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      const Mag<double> ov{__shfl_down_sync(0xffffffffu, best.hi, off),
+                      __shfl_down_sync(0xffffffffu, best.lo, off)};
+      const int oi = __shfl_down_sync(0xffffffffu, bi, off);
+      if (better(ov, oi, best, bi)) {
+        best = ov;
+        bi = oi;
+      }
+    }
+    if (lane == 0) {
+      const int pr = bi >= n ? j : bi;
+      pivot = perm[j] = pr;
+      recip = pivot_recip(A[pr * n + j], st);
+    }
+  };
+  if (wid == 0) search(0);
+  constexpr int kWorkers = kThreads - 32;
+  const int dr = kWorkers / n, dc = kWorkers - dr * n;
+  __syncthreads();
+  for (int j = 0; j < n; ++j) {
+    const int pr = pivot;
+    // row pr receives row j; the pivot row is kept scaled, row j itself is written with it below
+    if (tid < n) {
+      const z64 a = A[j * n + tid], v = A[pr * n + tid];
+      A[pr * n + tid] = a;
+      prow[tid] = tid == j ? recip : cmul(v, recip);
+      if (tid == j)
+        f[pr] = a;
+      else if (tid != pr)
+        f[tid] = A[tid * n + j];
+    }
+    __syncthreads();
+    if (wid == 0) {
+      const int c = j + 1;
+      if (c < n) {
+        const z64 pc = prow[c];
+        for (int r = lane; r < n; r += 32) {
+          z64 x = A[r * n + c];
+          eliminate(x, f[r], pc, other[r]);
+          A[r * n + c] = r == j ? pc : x;
+        }
+        __syncwarp();
+        search(c);
+      }
+    } else {
+      int r = (tid - 32) / n, c = tid - 32 - r * n;
+      while (r < n) {
+        if (c != j + 1) {
+          z64 x = c == j ? zero : A[r * n + c];
+          eliminate(x, f[r], prow[c], other[r]);
+          A[r * n + c] = r == j ? prow[c] : x;
+        }
+        r += dr;
+        c += dc;
+        if (c >= n) {
+          c -= n;
+          ++r;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    for (int c = 0; c < n; ++c) src[c] = c;
+    for (int j = n - 1; j >= 0; --j) {
+      int t = src[j];
+      src[j] = src[perm[j]];
+      src[perm[j]] = t;
+    }
+  }
+  __syncthreads();
+  z64* x = bat(X, p);
+  for (int r = 0; r < n; ++r)
+    for (int c = tid; c < n; c += kThreads) x[(long long)r * X.ld + c] = A[r * n + src[c]];
+}
+
 // Panel step of the blocked form: columns [k0, k0 + w) of A (n x n, in global memory).
 // The panel is eliminated in shared memory; then, for the columns outside the panel, one pass
 // per column (each column owned by one thread, so no barrier) moves the swapped rows to their
@@ -360,20 +501,6 @@ __global__ void __launch_bounds__(kThreads) k_gj_panel(int n, int k0, int w, int
 // that also moved the rows of the whole matrix took 110 us.  512 threads: 1024 spend more on the
 // part of a step that every warp repeats, and a test per slot (instead of filler rows) parted the
 // slots' loads and took 140 us.
-// The multiply-adds of a step are written out, each rounding in its place, so that the result does
-// not depend on how the compiler contracts them.  `other` takes the imaginary part's products in
-// the other order: the elimination has always done so in the rows that its unrolling by four left
-// over, and the results stay the same bit for bit.
-__device__ __forceinline__ cx<float> cmul(cx<float> a, cx<float> b) {
-  return mkc<float>(__fmaf_rn(a.re, b.re, -__fmul_rn(a.im, b.im)),
-                    __fmaf_rn(a.re, b.im, __fmul_rn(a.im, b.re)));
-}
-__device__ __forceinline__ void eliminate(cx<float>& x, cx<float> f, cx<float> p, bool other) {
-  x.re = __fsub_rn(x.re, __fmaf_rn(f.re, p.re, -__fmul_rn(f.im, p.im)));
-  const float t = other ? __fmaf_rn(f.re, p.im, __fmul_rn(f.im, p.re))
-                        : __fmaf_rn(f.im, p.re, __fmul_rn(f.re, p.im));
-  x.im = __fsub_rn(x.im, t);
-}
 // Pivot candidates.  hi + lo of mag2 is brought to h = RN(hi + lo) and the exact rest l, so that the
 // larger sum has the larger h, then the larger l; equal sums go to the lower row.  Keys order like
 // unsigned integers (a candidate's h key is at least 1), so a warp finds its winner with reductions
@@ -833,12 +960,10 @@ cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> 
   if (P <= 0 || n <= 0) return cudaSuccess;
   const int eb = (int)sizeof(z64);
   if (gj_fits_small(n, eb)) {
-    size_t smem = small_smem(n, eb);
-    cudaError_t e = cudaFuncSetAttribute(k_gj_small<double>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBudget + 1024);
+    cudaError_t e = cudaFuncSetAttribute(
+        k_gj_small64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 1024);
     if (e != cudaSuccess) return e;
-    k_gj_small<double><<<P, kThreads, smem, s>>>(n, M, X, status, active);
+    k_gj_small64<<<P, kThreads, small_smem(n, eb), s>>>(n, M, X, status, active);
     count_launch();
     return cudaGetLastError();
   }
