@@ -410,7 +410,7 @@ negf_status negf_zinv_batched_noalloc(int32_t n_batch, int32_t n, double* M, dou
  * 256-row MMA, stages released per MMA commit; K chunks of 64 per stage; 128-column tiles unless
  * stated) and splits K into at most (4, 8)[c % 2] exactly accumulated parts (more parts allow
  * wider slices and fewer slice products for long contractions).
- * negf_tc_config_set selects one process-wide (default 18: the CTA pair with 2 stages of 4 K
+ * negf_tc_config_set selects one process-wide (default 20: the CTA pair with 3 stages of 3 K
  * chunks); results agree to the GEMM's rounding.  The package's autotuner times them per block
  * size and stores the choice. */
 int32_t negf_tc_config_count(void);
@@ -420,8 +420,8 @@ int32_t negf_tc_config_get(void);
 /* ---- accounting ----------------------------------------------------------------------------
  * Instrumentation for benchmarks, not part of the method.  negf_launch_count() is the number
  * of kernels this library has launched since it was loaded.  With profiling on, every launch of
- * the tensor-core GEMM kernel (kind 0), of its operand slicing or residues (kind 1) and every Gauss-Jordan
- * elimination of a block inverse inside the sweeps (kind 2: the FP32 start of the mixed form or
+ * the tensor-core GEMM kernel (kind 0), of its operand slicing or residues (kind 1) and every
+ * Gauss-Jordan elimination of a block inverse inside the sweeps (kind 2: the FP32 start of the mixed form or
  * the whole FP64 inverse, without the Newton-Schulz products, which count as kinds 0 and 1) and
  * every launch of its panel-elimination kernel (kind 3, a part of kind 2) is
  * bracketed by CUDA events on its own stream; negf_profile_read synchronises those events and

@@ -656,7 +656,9 @@ constexpr TcShape kShapes[] = {{6, 1, 1, 128}, {6, 1, 2, 128}, {6, 1, 3, 128}, {
 // 96 KB).  Shapes 11-12: 64-column tiles (256 TMEM columns) with 2 stages of 2 K chunks, two
 // CTAs resident per SM so that one tile's waits and final pass overlap the other's MMAs.
 constexpr int kNumCfg = 2 * (int)(sizeof(kShapes) / sizeof(kShapes[0]));
-std::atomic<int> g_cfg{18};
+// The default, the CTA pair with 3 stages of 3 K chunks, serves calls of few items best (us, against 2
+// stages of 4 chunks: 1 x 1200^3 485 / 508, 2 x 800^3 366 / 379, 8 x 400^3 264 / 268, 4 x 340^3 151 / 150).
+std::atomic<int> g_cfg{20};
 
 bool tc_bits_ok(int bits) { return bits == 40 || bits == 48 || bits == 56; }
 
