@@ -19,7 +19,7 @@ struct Pending {
 };
 std::vector<Pending> g_pending;
 std::vector<cudaEvent_t> g_pool;
-cudaEvent_t g_open[PROF_KINDS] = {};
+thread_local cudaEvent_t g_open[PROF_KINDS] = {};  // begun by this thread
 long long g_count[PROF_KINDS] = {};
 double g_ms[PROF_KINDS] = {};
 double g_alg[PROF_KINDS] = {};

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from concurrent.futures import ThreadPoolExecutor
 from ctypes import POINTER, c_double, c_int32, c_size_t, c_void_p
 
 import torch
@@ -583,9 +584,10 @@ def solve_ragged(systems, opt: _Opt, outputs=("density", "current", "transmissio
         groups.setdefault((int(Hd.shape[0]), int(Hd.shape[1])), []).append(i)
     results = [None] * len(systems)
     cur = torch.cuda.current_stream()
+    modes = torch.is_grad_enabled(), torch.is_inference_mode_enabled()
     # the side streams are kept across calls: each owns a cached workspace
     pool = _RAGGED_STREAMS.setdefault(str(cur.device), [])
-    streams = []
+    jobs = []
     for g, ((N, b), idx) in enumerate(sorted(groups.items(), key=lambda kv: -kv[0][1])):
         if concurrent:
             while len(pool) <= g:
@@ -594,8 +596,12 @@ def solve_ragged(systems, opt: _Opt, outputs=("density", "current", "transmissio
         else:
             st = cur
         st.wait_stream(cur)
-        streams.append(st)
-        with torch.cuda.stream(st):
+        jobs.append((N, idx, st))
+
+    def solve(N, idx, st):
+        # the calling thread's device and modes, which a new thread does not have
+        with torch.inference_mode(modes[1]), torch.set_grad_enabled(modes[0]), \
+                torch.cuda.device(cur.device), torch.cuda.stream(st):
             Hd = torch.stack([systems[i][0] for i in idx])
             Hu = torch.stack([systems[i][1] for i in idx]) if N > 1 else None
             dev = Device(Hd, Hu)
@@ -611,7 +617,20 @@ def solve_ragged(systems, opt: _Opt, outputs=("density", "current", "transmissio
                 results[i] = {k: (v[off:off + n] if isinstance(v, torch.Tensor) else v)
                               for k, v in out.items()}
                 off += n
-    for st in streams:
+
+    # The decimation's host check waits for its stream every few steps, so one host thread would take
+    # the groups one after another; a thread per group lets their chains run side by side (the
+    # library calls release the interpreter lock).  Four sizes of b = 200 ... 800, 4 points:
+    # 330 -> 288 ms.
+    if concurrent and len(jobs) > 1 and opt.sr_host_check > 0:
+        library()  # loaded before the threads
+        with ThreadPoolExecutor(min(len(jobs), 16)) as ex:
+            for f in [ex.submit(solve, *job) for job in jobs]:
+                f.result()
+    else:
+        for job in jobs:
+            solve(*job)
+    for _, _, st in jobs:
         cur.wait_stream(st)
     return results
 
