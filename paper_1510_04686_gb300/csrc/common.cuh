@@ -124,21 +124,24 @@ inline cudaError_t launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_
 
 // ---- launchers (all asynchronous on `s`) ----------------------------------------------
 
+// Form of an FP64 product: chosen by size, or given.
+enum GemmForm { GEMM_AUTO = 0, GEMM_TILES = 1, GEMM_STRIPS = 2 };
 // C[p] = alpha op(A[p]) op(B[p]) + beta C[p] + gamma D[p] on the CUDA cores (FP64 form).
 // beta == 0 does not read C; D.p == NULL skips the D term.  Batch items with
 // active[p] == 0 are skipped (active may be NULL).
 cudaError_t gemm_simt(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
                       int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
-                      BMc<double> D, const int32_t* active);
+                      BMc<double> D, const int32_t* active, int form = GEMM_AUTO);
 
 // X[p] = M[p]^-1 by Gauss-Jordan elimination with partial pivoting (largest |m|, lowest row
 // on ties, pivots compared in FP64).  A zero pivot sets NEGF_PT_SINGULAR in status[p] and is
 // replaced by a tiny number so the sweep continues.  Scratch: piv (P x n).
-// FP64: M is destroyed; scratch U (P x n x nb), T (P x nb x n), nb = gj_panel_width(n, 16).
+// FP64: mostly_idle: active is expected to select no item.  M is destroyed; scratch U (P x n x nb), T (P x nb x n), nb = gj_panel_width(n, 16).
 // FP32: elimination in FP32 (m32 and x32: P x n x n, U: P x n x nb, nb = gj_panel_width(n, 8), map:
 // P x n), M is kept; M and X are contiguous n x n blocks.
 cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, z64* U, z64* T,
-                         int32_t* piv, int32_t* status, const int32_t* active);
+                         int32_t* piv, int32_t* status, const int32_t* active,
+                         bool mostly_idle = false);
 cudaError_t gj_inverse32(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, cx<float>* m32,
                          cx<float>* x32, cx<float>* U, int32_t* piv, int32_t* map, int32_t* status,
                          const int32_t* active);

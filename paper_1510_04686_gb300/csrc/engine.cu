@@ -213,7 +213,7 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(s, PROF_INV);
-  e = gj_inverse64(s, P, b, Mm, X, w.invU, w.invT, w.piv, status, w.act);
+  e = gj_inverse64(s, P, b, Mm, X, w.invU, w.invT, w.piv, status, w.act, true);
   prof_end(s, PROF_INV);
   return e;
 }

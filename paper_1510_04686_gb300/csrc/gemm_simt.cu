@@ -175,13 +175,22 @@ __global__ void __launch_bounds__(32 * kStripWarps)
 
 cudaError_t gemm_simt(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
                       int opA, BMc<double> B, int opB, z64 beta, BM<double> C, z64 gamma,
-                      BMc<double> D, const int32_t* active) {
+                      BMc<double> D, const int32_t* active, int form) {
   if (P <= 0 || M <= 0 || N <= 0) return cudaSuccess;
+  // Tiles run at the FP64 rate of an SM each, 64 x 64 x 4 multiply-adds per k step at two per clock, in
+  // waves of one per SM: 8192 clocks per k and wave.  Strips split evenly but reach 72 % of the rate.
+  // Measured, us, strips / tiles: 64 items of 40 36 / 166, 1 of 400 673 / 1686, 64 of 200 3380 / 5602, 3
+  // of 64 x 1000 x 500 1078 / 2107, 200 of 64 x 64 x 300 2245 / 2519; 64 of 128 1248 / 1090, 64 of 256
+  // 9503 / 7226, 64 of 400 36089 / 33482, 1 of 1200 15365 / 14448.  Both form the same sums.
   // Strips write their output while others still read: an output that starts on an operand goes to
-  // the tiles (right for it up to one tile), as does K = 0.  Measured, us, strips / tiles: b = 40,
-  // 1 item 8.7 / 166, 64 items 36 / 166; b = 64, 64 items 124 / 265, 512 items 943 / 1043; b = 128,
-  // 64 items 904 / 1036, 512 items 7181 / 7181; b = 200, 64 items 3380 / 5602.
-  if (K > 0 && C.p != A.p && C.p != B.p) {
+  // the tiles (right for it up to one tile), as does K = 0.
+  constexpr long long kSms = 152;
+  const long long tiles = (long long)((M + BMT - 1) / BMT) * ((N + BNT - 1) / BNT) * P;
+  const double tile_clocks = 8192.0 * ((tiles + kSms - 1) / kSms);
+  const double strip_clocks = 2.0 / 0.72 / kSms * P * ((M + kStripRows - 1) / kStripRows * kStripRows) *
+                              ((N + kStripCols - 1) / kStripCols * kStripCols);
+  const bool strips = form == GEMM_AUTO ? strip_clocks < tile_clocks : form == GEMM_STRIPS;
+  if (strips && K > 0 && C.p != A.p && C.p != B.p) {
     const long long strips =
         (long long)((M + kStripRows - 1) / kStripRows) * ((N + kStripCols - 1) / kStripCols);
     // CTAs per item: enough to fill the chip, few enough that masked items cost little

@@ -953,10 +953,11 @@ cudaError_t panel32(cudaStream_t s, int P, int n, int k0, int w, int nb, const c
 
 // Both eliminations are chains of two short kernels per panel, and the mixed form's FP64 fallback runs
 // its whole chain without an item in nearly every call: the kernels are launched chained, which took
-// the inverse of one 400 block from 1782 to 1586 us, of one 2400 block from 39.5 to 31.6 ms, of 64
-// blocks of 400 from 5.57 to 5.44 ms.
+// the inverse of one 400 block (mixed) from 1782 to 1586 us, of one 2400 block from 39.5 to 31.6 ms, of 64
+// blocks of 400 from 5.57 to 5.44 ms.  The update is a chained product by strips there; with items to
+// work on it is one by tiles, not chained (64 FP64 blocks of 400: 45.0 ms, 48.7 chained, 50.5 by strips).
 cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> X, z64* U, z64* T,
-                         int32_t* piv, int32_t* status, const int32_t* active) {
+                         int32_t* piv, int32_t* status, const int32_t* active, bool mostly_idle) {
   if (P <= 0 || n <= 0) return cudaSuccess;
   const int eb = (int)sizeof(z64);
   if (gj_fits_small(n, eb)) {
@@ -985,7 +986,7 @@ cudaError_t gj_inverse64(cudaStream_t s, int P, int n, BM<double> M, BM<double> 
     BMc<double> Ta{T, (long long)nb * n, nullptr, n};
     BMc<double> none{nullptr, 0, nullptr, 0};
     e = gemm_simt(s, P, n, n, w, mkc<double>(1.0, 0.0), Ua, OP_N, Ta, OP_N, mkc<double>(1.0, 0.0),
-                  M, mkc<double>(0.0, 0.0), none, active);
+                  M, mkc<double>(0.0, 0.0), none, active, mostly_idle ? GEMM_STRIPS : GEMM_TILES);
     if (e != cudaSuccess) return e;
   }
   // T is free again
