@@ -422,7 +422,9 @@ def zgemm(A, B, C=None, alpha=1.0, beta=0.0, opA="N", opB="N", precision=PREC_FP
     if K != K2:
         raise ValueError("inner dimensions differ")
     if C is None:
-        C = torch.zeros((nb, M, N), dtype=torch.complex128, device=A.device)
+        # a product that does not accumulate writes every entry
+        make = torch.empty if beta == 0 else torch.zeros
+        C = make((nb, M, N), dtype=torch.complex128, device=A.device)
     _need(C, torch.complex128, "C", (nb, M, N))
     ws_n = int(library().negf_zgemm_workspace_size(precision, nb, M, N, K))
     ws = _workspace(ws_n, A.device)
