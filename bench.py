@@ -31,13 +31,10 @@ WORK = dict(N=70, b=400, n_E=512, n_k=8, ge_frac=0.1, eta=1e-6, seed=1001,
             name="ballistic RGF, N=70 slabs x 400x400 blocks, alloy p(Ge)=0.1, 512 E x 8 k")
 METRIC = "RGF energy-points/s (leads + forward/backward sweeps + observables + FP64 quadrature)"
 PEAKS_FALLBACK = dict(hbm_gbs=6800.0, bf16_tflops=1900.0, bf16_tflops_sustained=1700.0)
-# DRAM bytes (read + write) of k_tc_gemm per 400 x 400 x 400 complex item from an ncu capture of
-# a 64-item 48-bit launch of tensor-core configuration 18 (820.4 MB read + 149.1 MB written),
-# scaled by the items of a launch; None once the kernel has changed since the capture (the line
-# then reports null).
-TC_DRAM_BYTES_PER_ITEM_B400 = (820.392448e6 + 149.107456e6) / 64
-# configurations 18 and 19 run the same launch at b = 400 (one K part under either policy)
-TC_PROFILED_CONFIGS = (18, 19)
+# DRAM bytes (read + write) of k_crt_gemm per 400 x 400 x 400 complex item from an ncu capture of
+# a 64-item 48-bit launch (1015.4 MB read + 159.8 MB written), scaled by the items of a launch; None
+# once the kernel has changed since the capture (the line then reports null).
+TC_DRAM_BYTES_PER_ITEM_B400 = (1015.397e6 + 159.823e6) / 64
 GOLDEN = os.path.join(ROOT, "tests", "golden", "c1_oracle.json")
 
 
@@ -332,7 +329,7 @@ def run_side(args):
         ms, _ = _timed(torch, born, args.warmup, args.steps)
         line.update(metric="SCBA point-iterations/s (RGF with phonon self-energies + Born update)",
                     value=nE * args.steps / (ms / 1e3), unit="point-iterations/s",
-                    ms_per_step=ms / args.steps, dtype="bf16-slices->fp32 (fp64 storage)",
+                    ms_per_step=ms / args.steps, dtype="bf16-integers->fp32 (fp64 storage)",
                     config={"workload": f"SCBA N=70 b=600, energies 0..{nE - 1} of the 5 meV grid, "
                                         + ("atom-block (10 x 10) self-energies" if atom else
                                            "orbital-diagonal self-energies"),
@@ -390,7 +387,7 @@ def run_side(args):
                             if args.adj_ckpt else
                             "adjoint points/s (forward sweep kept + reverse sweep, dL/dV)"),
                     value=args.steps / (ms / 1e3), unit="points/s", ms_per_step=ms / args.steps,
-                    dtype="bf16-slices->fp32 (fp64 storage)",
+                    dtype="bf16-integers->fp32 (fp64 storage)",
                     config={"workload": f"adjoint, N={N} slabs x 3430 orbitals (343 atoms x 10),"
                                         " V ~ U(-0.3, 0.3) eV per atom, 1 point"
                                         + (f", hoppings on the {args.adj_iface} x "
@@ -432,7 +429,7 @@ def run_side(args):
         line.update(metric="energy-points/s with interface couplings (lead decimation + RGF "
                            "sweeps)",
                     unit="points/s", value=it["step"], ms_per_step=it["ms"],
-                    dtype="bf16-slices->fp32 (fp64 storage)",
+                    dtype="bf16-integers->fp32 (fp64 storage)",
                     config={"workload": f"N=70 slabs x 400x400 blocks, hoppings between the "
                                         f"{r // 10} facing atoms of each slab ({r} x {c} support),"
                                         f" {P} points",
@@ -459,7 +456,7 @@ def run_side(args):
         res = (torch.eye(b, dtype=torch.complex128, device=dvc) - M0 @ X).abs().max().item()
         line.update(metric="batched block inverses/s (mixed: FP32 Gauss-Jordan + Newton-Schulz)",
                     value=nb * args.steps / (ms / 1e3), unit="inverses/s",
-                    ms_per_step=ms / args.steps, dtype="fp32 elimination, bf16-slices->fp32 "
+                    ms_per_step=ms / args.steps, dtype="fp32 elimination, bf16-integers->fp32 "
                     "refinement (fp64 in/out)",
                     config={"workload": f"{nb} items of {b} x {b} complex128",
                             "max_residual": res,
@@ -481,7 +478,7 @@ def run_side(args):
         n_sl, sl_ms, _, _ = negf.profile_read(negf.PROF_SLICE)
         line.update(metric="batched complex GEMM, algorithmic TFLOP/s (8 b^3 per item)",
                     value=8.0 * b ** 3 * nb * args.steps / (ms / 1e3) / 1e12, unit="TFLOP/s",
-                    ms_per_step=ms / args.steps, dtype="bf16-slices->fp32 (fp64 in/out)",
+                    ms_per_step=ms / args.steps, dtype="bf16-integers->fp32 (fp64 in/out)",
                     config={"workload": f"{nb} items of {b} x {b} x {b} complex128",
                             "tc_config": negf.tc_config(),
                             "tc_kernel_ms": tc_ms / max(n_tc, 1),
@@ -520,7 +517,7 @@ def run_side(args):
                     for b, x in zip(bs, systems))
         line.update(metric="RGF energy-points/s over ragged block sizes (one CUDA graph)",
                     unit="points/s", value=n_pts * args.steps / (ms / 1e3),
-                    ms_per_step=ms / args.steps, dtype="bf16-slices->fp32 (fp64 storage)",
+                    ms_per_step=ms / args.steps, dtype="bf16-integers->fp32 (fp64 storage)",
                     config={"workload": f"{n_s} samples of the b = 200..800 alloy set (N = 70), "
                                         f"4 k-points x {n_e} energies each: {n_pts} points",
                             "systems_per_block_size": counts,
@@ -639,7 +636,7 @@ def main():
     peak_bf16 = pk.get("bf16_tflops_sustained", PEAKS_FALLBACK["bf16_tflops_sustained"])
     achieved = (alg / (tc_ms / 1e3)) / 1e12 if tc_ms > 0 else None
     roofline = {
-        "kernel": "k_tc_gemm (tcgen05 split-BF16 complex GEMM)",
+        "kernel": "k_crt_gemm (tcgen05 complex GEMM on BF16 residues)",
         "bound": "tensor", "unit": "TFLOP/s",
         "achieved": achieved, "peak": peak_bf16,
         "frac": (achieved / peak_bf16) if achieved else None,
@@ -654,8 +651,7 @@ def main():
         "gj_panel_share_of_step": pan_ms / ms if ms > 0 else None,
         "traffic": (TC_DRAM_BYTES_PER_ITEM_B400 * (alg / max(n_launch, 1)) / (8.0 * WORK["b"] ** 3)
                     if TC_DRAM_BYTES_PER_ITEM_B400 and WORK["b"] == 400 and n_launch
-                    and prec == negf.PREC_MIXED and negf.tc_config() in TC_PROFILED_CONFIGS
-                    else None),
+                    and prec == negf.PREC_MIXED else None),
         "traffic_unit": "bytes per launch (DRAM read + write, ncu capture of 64 items scaled "
                         "to the launch's items)",
     }
@@ -663,7 +659,7 @@ def main():
         "metric": METRIC, "value": value, "unit": "points/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": (f"bf16-slices->fp32 (fp64 storage; sweeps {tier_bits(negf, prec)}-bit, "
+        "dtype": (f"bf16-integers->fp32 (fp64 storage; sweeps {tier_bits(negf, prec)}-bit, "
                   "lead decimation 56/48/40-bit by doubling step)") if mixed else "f64",
         "data": "synthetic",
         "config": {"workload": WORK["name"], "points_per_step": P, "precision": args.precision,
