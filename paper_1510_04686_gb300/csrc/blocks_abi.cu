@@ -58,7 +58,7 @@ negf_status negf_zgemm_batched(int32_t precision, int32_t n_batch, int32_t M, in
     const int bits = prec_bits(precision);
     if (residue_products(n_batch)) {
       CrtWs cw;
-      crt_ws_carve(base, off, n_batch, M, N, K, bits, cw);
+      crt_ws_carve(base, off, n_batch, M, N, K, bits, false, cw);
       e = crt_gemm(s, n_batch, M, N, K, al, a, opA, b, opB, be, c, zero, none, false, nullptr, cw,
                    bits);
     } else {

@@ -545,7 +545,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ------------------------------------------------------------------ host side
-inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 inline int ceil_div(int x, int m) { return (x + m - 1) / m; }
 
 struct GemmArgs {
@@ -645,40 +644,27 @@ cudaError_t crt_prof_reset() {
 size_t crt_ws_bytes(int P, int M, int N, int K, int bits) {
   size_t off = 0;
   CrtWs w;
-  crt_ws_carve(nullptr, off, P, M, N, K, bits, w);
+  crt_ws_carve(nullptr, off, P, M, N, K, bits, false, w);
   return off;
 }
 
-// Row length of the residue planes: K rounded up to 8 (rows of whole 16-byte units for the TMA).
-static int residue_ld(int K) { return round_up(K, 8); }
-
-// Most moduli of a plan for any contraction up to K (products of a block's parts share the
-// workspace of the whole block).
-static int most_moduli(int K, int bits) {
-  int n = 0;
-  CrtPlan pl;
-  for (int k : {K, std::min(K, 256), std::min(K, 400), std::min(K, 512), std::min(K, 640),
-                std::min(K, 800), std::min(K, 1024), std::min(K, 1025)})
-    if (crt_plan(k, bits, &pl)) n = std::max(n, pl.n);
-  return n;
-}
-
-void crt_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits, CrtWs& w) {
-  // a product may take a narrower tier than the one that the scratch is for
-  int most = 0;
-  for (int t : {40, 48, 56})
-    if (t <= bits) most = std::max(most, most_moduli(K, t));
-  const size_t n = (size_t)most, L = (size_t)residue_ld(K);
+void crt_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits, bool shorter,
+                  CrtWs& w) {
+  const size_t line = crt_line_elements(K, bits, shorter);
   auto take = [&](size_t bytes) -> void* {
     size_t a = (off + 1023) & ~size_t(1023);
     off = a + bytes;
     return base ? base + a : nullptr;
   };
+  w.linesA = (size_t)P * M;
+  w.linesB = (size_t)P * N;
+  w.elemsA = w.linesA * line;
+  w.elemsB = w.linesB * line;
   w.err = static_cast<int32_t*>(take(256));  // first, so that its place does not depend on P
-  w.resA = take((size_t)P * 2 * n * M * L * 2);
-  w.resB = take((size_t)P * 2 * n * N * L * 2);
-  w.expA = static_cast<int32_t*>(take((size_t)P * M * 4));
-  w.expB = static_cast<int32_t*>(take((size_t)P * N * 4));
+  w.resA = take(w.elemsA * 2);
+  w.resB = take(w.elemsB * 2);
+  w.expA = static_cast<int32_t*>(take(w.linesA * 4));
+  w.expB = static_cast<int32_t*>(take(w.linesB * 4));
 }
 
 cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,
@@ -712,6 +698,10 @@ cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<
   if (!crt_plan(K, bits, &g.plan))
     return cudaErrorInvalidValue;  // K beyond the tier's range (callers check tc_supports_k)
   const int L = residue_ld(K);
+  const size_t line = 2 * (size_t)g.plan.n * L, linesA = (size_t)PA * M, linesB = (size_t)PB * N;
+  if (linesA > ws.linesA || linesB > ws.linesB || linesA * line > ws.elemsA ||
+      linesB * line > ws.elemsB)
+    return cudaErrorInvalidValue;
   __nv_bfloat16* ra = static_cast<__nv_bfloat16*>(ws.resA);
   __nv_bfloat16* rb = static_cast<__nv_bfloat16*>(ws.resB);
   const KeptOperand ka{A.p,  ra,  g.zA ? g.zA : A.idx, actA, A.stride,   A.ld,

@@ -25,12 +25,16 @@ struct CrtWs {
   int32_t* expA;        // [P][M]
   int32_t* expB;        // [P][N]
   int32_t* err;         // device error word (bounded waits that gave up)
+  size_t elemsA, elemsB;  // what resA and resB hold, and the lines of expA and expB: a product
+  size_t linesA, linesB;  // that needs more is refused
 };
 
-// Bytes of CrtWs scratch for P items of an M x N x K product (or any shorter contraction) at
-// `bits` bits per value.
+// CrtWs scratch for P items of an M x N x K product at `bits` bits per value; with `shorter`, for
+// every product of up to K terms at these bits or fewer, as the sweeps of b x b blocks need it.
+void crt_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits, bool shorter,
+                  CrtWs& w);
+// Bytes of the scratch of one product.
 size_t crt_ws_bytes(int P, int M, int N, int K, int bits);
-void crt_ws_carve(char* base, size_t& off, int P, int M, int N, int K, int bits, CrtWs& w);
 
 // Flops of the tensor-core GEMM launches made while profiling was on, counted on the device
 // for the items that ran (the current device; both calls synchronise it): algorithmic complex
@@ -40,7 +44,7 @@ cudaError_t crt_prof_reset();
 
 // n_distinct: number of different matrices an indexed operand (idx != NULL) selects from
 // (0 = unknown: convert every item).  bits: fixed-point bits per operand value (tc_bits_ok); the
-// workspace must have been carved for these bits or more.  rmax (nullable, float [P], zeroed by the
+// workspace must have been carved for such a product (else cudaErrorInvalidValue).  rmax (nullable, float [P], zeroed by the
 // caller): rmax[p] is raised to the largest |Re| or |Im| of item p's outputs (the Newton-Schulz
 // residual norm when C = I - M X).  kept (nullable): what the scratch of `ws` holds, see Kept.
 cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<double> A,

@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include "tc_gemm.cuh"
 
@@ -179,6 +180,26 @@ bool crt_plan(int K, int bits, CrtPlan* out) {
     *out = CrtPlan{c, n, parts, per, (sum + 1) / 2, sum / 2, bits == 56};
   }
   return best >= 0.0;
+}
+
+size_t crt_line_elements(int K, int bits, bool shorter) {
+  if (!shorter) {
+    CrtPlan pl;
+    return crt_plan(K, bits, &pl) ? 2 * (size_t)pl.n * residue_ld(K) : 0;
+  }
+  // running maxima over k, extended as far as they have been asked for
+  static std::mutex mu;
+  static std::vector<size_t> most[3];
+  constexpr int kTiers[3] = {40, 48, 56};
+  std::lock_guard<std::mutex> lk(mu);
+  size_t need = 0;
+  for (int t = 0; t < 3 && kTiers[t] <= bits; ++t) {
+    std::vector<size_t>& m = most[t];
+    for (int k = (int)m.size() + 1; k <= K; ++k)
+      m.push_back(std::max(m.empty() ? 0 : m.back(), crt_line_elements(k, kTiers[t], false)));
+    need = std::max(need, m[K - 1]);
+  }
+  return need;
 }
 
 const ResidueConst& residue_const(const CrtPlan& pl) {

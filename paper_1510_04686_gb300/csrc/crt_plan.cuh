@@ -8,6 +8,7 @@
 // One complex product modulo p is then two real products u u', v v' (instead of the four of a
 // real embedding), and Re = (u + v) / 2, Im = (u - v) / (2 j).
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 
 namespace negf {
@@ -59,6 +60,13 @@ struct CrtPlan {
 // The plan for a contraction of K complex terms at `bits` bits per value; false where the tier
 // does not cover K (tc_supports_k).
 bool crt_plan(int K, int bits, CrtPlan* out);
+// Row length of the residue planes: K rounded up to 8 (rows of whole 16-byte units for the TMA).
+inline int residue_ld(int K) { return (K + 7) / 8 * 8; }
+// Elements of one operand line in all residue planes of a contraction of K terms (2 n rows); with
+// `shorter`, the most that any contraction of up to K terms takes in this tier or a narrower one.
+// The number of moduli does not grow with K: 513 to 560 terms in the 48-bit tier take 13 in one K
+// part, 561 to 600 take 12 in two, so the longest contraction is not always the one that needs most.
+size_t crt_line_elements(int K, int bits, bool shorter);
 // Constants of a plan's modulus set (its first n moduli).
 const ResidueConst& residue_const(const CrtPlan& pl);
 const CrtConst& crt_const(const CrtPlan& pl);

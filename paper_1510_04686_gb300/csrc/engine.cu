@@ -65,7 +65,7 @@ void carve_engine(char* base, size_t& off, int P, int b, int precision, bool res
     off = a;
     if (residues) {
       CrtWs cw;
-      crt_ws_carve(base, off, P, b, b, b, prec_bits(precision), cw);
+      crt_ws_carve(base, off, P, b, b, b, prec_bits(precision), true, cw);
     } else {
       TcWs tw;
       tc_ws_carve(base, off, P, b, b, b, prec_bits(precision), tw);
@@ -107,7 +107,7 @@ static TcWs tc_view(const EngineWs& w, int P, int b, int bits) {
 static CrtWs crt_view(const EngineWs& w, int P, int b, int bits) {
   CrtWs t;
   size_t off = 0;
-  crt_ws_carve(static_cast<char*>(w.tc), off, P, b, b, b, bits, t);
+  crt_ws_carve(static_cast<char*>(w.tc), off, P, b, b, b, bits, true, t);
   return t;
 }
 // The device error word, first in the operand scratch of either form.
