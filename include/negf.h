@@ -76,10 +76,11 @@ typedef enum {
  * op(A) and column of op(B) is scaled by a power of two and rounded once to fixed point (the
  * tiers are named 40, 48 and 56 bits), and the fixed-point product is formed exactly from BF16
  * operands; storage, pivoting, norms and reductions stay FP64.  Calls of 12 points (batch items)
- * or more form it modulo 10-14 small integers (residue products): a product's error is about
- * 2^-(bits + 2) x |row of A| x |column of B| (2-norms), that of an FP64 product in the 56-bit
- * tier, and a complex product issues 20 (40 bits), 24 (48 bits) or 28 (56 bits) real products at
- * 257-400 contracted terms.  Calls of fewer points cut the values into BF16 slices: the error is
+ * or more form it modulo 10-15 small integers (residue products): a product's error is usually a
+ * quarter of 2^-bits x |row of A| x |column of B| (2-norms) and stays below that unless its
+ * roundings are equal term by term (lines of equal entries); in the 56-bit tier it is that of an
+ * FP64 product.  A complex product issues 20 (40 bits), 24 (48 bits) or 28 (56 bits) real products
+ * at 257-400 contracted terms.  Calls of fewer points cut the values into BF16 slices: the error is
  * about 2^-bits x K x max|row of A| x max|column of B|, for 60, 84 or 112 real products. */
 typedef enum {
   NEGF_PREC_FP64 = 0,     /* every block operation in FP64 on the CUDA cores (reference form) */

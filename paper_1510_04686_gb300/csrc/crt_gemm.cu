@@ -725,7 +725,7 @@ cudaError_t crt_gemm(cudaStream_t s, int P, int M, int N, int K, z64 alpha, BMc<
   count_launch(!haveA + !haveB);
   if (e != cudaSuccess) return e;
   if (kept) *kept = Kept{ka, kb, 0};
-  // the 56-bit tier's fractions carry correction sums, whose registers limit the tile to 64
+  // correction sums of the fractions: their registers limit the tile to 64
   const bool hp = g.plan.hp;
   const int nt = pick_width(P, M, N, hp);
   g.resA = ra;

@@ -43,7 +43,7 @@ cudaError_t crt_prof_flops(double* alg, double* hw);
 cudaError_t crt_prof_reset();
 
 // n_distinct: number of different matrices an indexed operand (idx != NULL) selects from
-// (0 = unknown: convert every item).  bits: fixed-point bits per operand value (tc_bits_ok); the
+// (0 = unknown: convert every item).  bits: a tier's (tc_bits_ok) or kCorrectionBits; the
 // workspace must have been carved for such a product (else cudaErrorInvalidValue).  rmax (nullable, float [P], zeroed by the
 // caller): rmax[p] is raised to the largest |Re| or |Im| of item p's outputs (the Newton-Schulz
 // residual norm when C = I - M X).  kept (nullable): what the scratch of `ws` holds, see Kept.

@@ -143,32 +143,46 @@ void build() {
 
 void ready() { std::call_once(g_once, build); }
 
-// log2 P that a tier needs.  A product's rounding error is about 2^-(alpha + 0.8) of
-// |A line| |B line| (2-norms) with 2 alpha = log2 P - 1 or more; the thresholds put it at or
-// below that of fixed-point digit products of the tier's width (for 48-bit values and K = 400,
-// measured, 2^-48.2 of the norms), with the wider digit values such products need beyond
-// K = 1024.  The 56-bit tier's products are at the level of FP64 arithmetic or below.
-double need_bits(int K, int bits) {
-  if (bits == 40) return K <= 1024 ? 81.0 : 88.0;
-  if (bits == 48) return K <= 256 ? 97.0 : (K <= 1024 ? 98.0 : 101.5);
-  return 114.0;
+// Least alpha_a + alpha_b of a tier of w-bit values (tc_value_bits, those of the digit products).  A
+// line is scaled so that its 2-norm lies in [2^(alpha - 1), 2^alpha); the roundings of both operands
+// then put a result off by 1.2 * 2^-alpha |A line| |B line| (rms) at most, and alpha = w + 2 holds
+// nearly all results within 2^-w |A line| |B line|.  Digit products, whose values are rounded relative
+// to the largest entry of a line, are stated to 2^-w K max|A line| max|B line|, which is never less.
+// Error against 64 bits, relative to the result, here / digits: normally distributed entries, 48 bits,
+// K = 400 1.4e-14 / 4.9e-14, 512 3.8e-15 / 5.1e-14, 1024 2.8e-14 / 6.2e-14; 40 bits, K = 512
+// 9.1e-13 / 1.2e-11.  Entries of one size, the most favourable to digits: 48 bits, K = 400 1.4e-14 /
+// 6.9e-15, 512 3.8e-15 / 6.9e-15, 1024 2.8e-14 / 7.1e-15; one modulus more would bring these level too,
+// for 733 -> 857 us of 64 products of 400^3.
+// The 56-bit tier is at the level of FP64 arithmetic, below its digit products.  Corrections: 2^-40 of
+// |A line| |B line| (2^-43 for the longest), so that a product with |B| <= 2^-24 everywhere is good to
+// 2^-58 of |A line|.  (40-bit contractions beyond 1024 terms take nearly what the wider digits of the
+// longest ones, 42 bits, ask for.)
+int need_alpha(int K, int bits) {
+  if (bits == 56) return 113;
+  if (bits == kCorrectionBits) return K <= 1024 ? 80 : 87;
+  const int need = 2 * tc_value_bits(K, bits) + 4;
+  return bits == 40 && K > 1024 ? std::max(need, 87) : need;
 }
+// Whether the rounding of the reconstruction's fractions to 64 bits would show: it is about 2^-67 p
+// sqrt(n parts) of P, half of what the 48-bit tier allows at some 5000 terms.
+bool need_corrections(int K, int bits) { return bits == 56 || (bits == 48 && K > 4096); }
 
 }  // namespace
 
 bool crt_plan(int K, int bits, CrtPlan* out) {
-  if (!tc_supports_k(K, bits)) return false;
+  if (!tc_supports_k(K, std::max(bits, 40))) return false;
   ready();
   // Cost of a plan in K terms of one real product per output: n moduli, each with one
   // accumulator flush per part that is worth kFlush terms (the flush of one part overlaps the
   // products of the next), plus the residues of both operands.
   constexpr double kFlush = 320.0, kResidue = 0.5;
   const int k16 = (K + 15) / 16;
+  const int need = need_alpha(K, bits);
   double best = -1.0;
   for (int c = 0; c < kClasses; ++c) {
     const Class& k = g_class[c];
     int n = 1;
-    while (n <= k.count && k.log2P[n] < need_bits(K, bits)) ++n;
+    while (n <= k.count && std::min(k.alpha[n], 2 * kMaxAlpha) < need) ++n;
     if (n > k.count) continue;
     const int most = kClassK[c] / 16;
     const int parts = (k16 + most - 1) / most;
@@ -177,7 +191,7 @@ bool crt_plan(int K, int bits, CrtPlan* out) {
     if (best >= 0.0 && cost >= best) continue;
     best = cost;
     const int sum = std::min(k.alpha[n], 2 * kMaxAlpha);
-    *out = CrtPlan{c, n, parts, per, (sum + 1) / 2, sum / 2, bits == 56};
+    *out = CrtPlan{c, n, parts, per, (sum + 1) / 2, sum / 2, need_corrections(K, bits)};
   }
   return best >= 0.0;
 }
@@ -189,11 +203,11 @@ size_t crt_line_elements(int K, int bits, bool shorter) {
   }
   // running maxima over k, extended as far as they have been asked for
   static std::mutex mu;
-  static std::vector<size_t> most[3];
-  constexpr int kTiers[3] = {40, 48, 56};
+  static std::vector<size_t> most[4];
+  constexpr int kTiers[4] = {kCorrectionBits, 40, 48, 56};
   std::lock_guard<std::mutex> lk(mu);
   size_t need = 0;
-  for (int t = 0; t < 3 && kTiers[t] <= bits; ++t) {
+  for (int t = 0; t < 4 && kTiers[t] <= bits; ++t) {
     std::vector<size_t>& m = most[t];
     for (int k = (int)m.size() + 1; k <= K; ++k)
       m.push_back(std::max(m.empty() ? 0 : m.back(), crt_line_elements(k, kTiers[t], false)));

@@ -31,11 +31,11 @@ struct ResidueConst {
 // Im x / P = sum_l t_l im[l] modulo 1, both as 64-bit binary fractions (the wrap-around of the
 // integer sum is the reduction modulo 1).  hre, him: what the rounding of re[l], im[l] to 64 bits
 // left, in units of the last place; their sums correct the fraction where its own rounding would
-// show (the 56-bit tier: it is 2^-56.6 of P, the operands' rounding 2^-60).  P = sigma 2^expo with sigma in (1/2, 1): the values of
+// show (CrtPlan::hp; in the 56-bit tier it is 2^-56.6 of P, the operands' rounding 2^-60).  P = sigma 2^expo with sigma in (1/2, 1): the values of
 // op(A) are multiplied by sigma before they are rounded to integers, so that the product itself is
 // simply fraction * 2^expo (a multiplication per operand value instead of one per result, which
-// would stand at the end of every tile).  The 56-bit tier, whose operands would feel the rounding of that
-// multiplication, multiplies the results by mant instead.
+// would stand at the end of every tile).  Where the fractions are corrected the results are multiplied
+// by mant instead: the 56-bit tier's operands would feel the rounding of that multiplication.
 struct CrtConst {
   float invp[kMaxMod];
   float negp[kMaxMod];
@@ -54,11 +54,13 @@ struct CrtPlan {
   int k16;         // 16-wide K steps per part (the last part may be shorter)
   int alpha_a;     // line norms of op(A) are scaled below 2^alpha_a,
   int alpha_b;     // those of op(B) below 2^alpha_b; 2^(alpha_a + alpha_b) < P / 2
-  bool hp;         // the fractions need their correction sums (56-bit tier)
+  bool hp;         // the fractions need their correction sums (56-bit tier, long contractions)
 };
 
-// The plan for a contraction of K complex terms at `bits` bits per value; false where the tier
-// does not cover K (tc_supports_k).
+// Products inside the refinement of an inverse (engine.cu), which need no tier's precision.
+constexpr int kCorrectionBits = 36;
+// The plan for a contraction of K complex terms at `bits` bits per value (a tier's, or
+// kCorrectionBits); false where the tier does not cover K (tc_supports_k).
 bool crt_plan(int K, int bits, CrtPlan* out);
 // Row length of the residue planes: K rounded up to 8 (rows of whole 16-byte units for the TMA).
 inline int residue_ld(int K) { return (K + 7) / 8 * 8; }

@@ -182,19 +182,18 @@ cudaError_t Engine::inv(int P, BM<double> Mm, BM<double> X, int32_t* status,
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const z64 zero = mkc(0.0, 0.0), one = mkc(1.0, 0.0), mone = mkc(-1.0, 0.0);
     if (w.residues) {
-      // A step that every item follows with another one needs its residual to 40 bits only: that
-      // error, 2^-40 |M| |X| in R, is the next step's to remove, as is R^2 (an FP32 start leaves
-      // R = 2^-24 |M| |X| or more, so no item takes a step more for it).  The correction X R needs
-      // 40 bits always: an item is done when |R| <= 2^-24, where they put the error of X R below
-      // 2^-59 of |X|.  64 blocks of 400 in the 48-bit tier: 5.93 -> 5.74 ms, 32 in the 56-bit tier
-      // 4.27 -> 3.88 ms, same error against 64 bits (6.0e-13, 1.6e-13).
+      // A step that every item follows with another one does not need its residual in the tier's
+      // precision: the error of kCorrectionBits, 2^-40 |M| |X| in R, is the next step's to remove,
+      // as is R^2 (an FP32 start leaves R = 2^-24 |M| |X| or more, so no item takes a step more for
+      // it).  The correction X R needs no more at any step: an item is done when |R| <= 2^-24, where
+      // they put the error of X R below 2^-58 of |X|.
       const CrtWs cw = crt_view(w, P, b, bits);
-      const int rbits = it + 1 < refine_min ? 40 : bits;
+      const int rbits = it + 1 < refine_min ? kCorrectionBits : bits;
       e = crt_gemm(s, P, b, b, b, mone, Mc, OP_N, Xc, OP_N, zero, R, zero, none, true, w.act, cw,
                    rbits, 0, w.rmax);
       if (e != cudaSuccess) return e;
       e = crt_gemm(s, P, b, b, b, one, Xc, OP_N, cst(R), OP_N, zero, X, one, Xc, false, w.act, cw,
-                   40);
+                   kCorrectionBits);
       if (e != cudaSuccess) return e;
       continue;
     }

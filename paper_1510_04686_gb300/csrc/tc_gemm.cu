@@ -709,6 +709,11 @@ bool tc_supports_k(int K, int bits) {
   return K >= 1 && tc_plan(K, bits, 4, &pl) && tc_plan(K, bits, 8, &pl);
 }
 
+int tc_value_bits(int K, int bits) {
+  TcPlan pl;
+  return tc_plan(K, bits, 4, &pl) ? pl.beta * pl.S : bits;
+}
+
 
 namespace {
 __global__ void k_flag_timeout(const int32_t* err, int P, int32_t* status) {

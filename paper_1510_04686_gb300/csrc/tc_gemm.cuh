@@ -66,6 +66,9 @@ bool tc_plan(int K, int bits, int max_parts, TcPlan* out);
 // Whether the tensor-core GEMM covers K exactly under every configuration at `bits` bits per
 // value (48 bits: K <= 28032).
 bool tc_supports_k(int K, int bits);
+// Bits per operand value of these products for K terms under the default K-part policy: `bits`, or
+// the whole digits above it (48-bit values take 6 digits of 8 bits, or 7 of 7 in long contractions).
+int tc_value_bits(int K, int bits);
 
 // The device error word ws.err is set when a bounded wait inside the GEMM kernel gave up (the
 // tile's outputs are then NaN).  tc_timeout_reset zeroes it; tc_timeout_flag ORs

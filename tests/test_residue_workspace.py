@@ -11,11 +11,11 @@ def test_scratch_of_a_block_holds_every_shorter_contraction(prec, n):
     negf._build.build()
     lib = negf.library()
     gemm, inv = lib.negf_zgemm_workspace_size, lib.negf_zinv_workspace_size
-    slack = 8 * 1024  # alignment of the pieces
+    slack = 64 * 1024  # alignment of the pieces
     for b in (*range(8, 520, 37), *range(520, 660), *range(660, 2000, 61), 3430, 9266):
-        # what a block operation needs beside its operands' residues is the same in every tier, and
-        # the 40-bit tier's residues never grow with fewer terms
-        rest = inv(negf.PREC_MIXED_40, n, b) - gemm(negf.PREC_MIXED_40, n, b, b, b)
+        # what an inverse needs beside its products' operands grows with the number of blocks; eleven
+        # blocks take digit slices, whose scratch never grows with fewer terms
+        rest = (inv(prec, 11, b) - gemm(prec, 11, b, b, b)) * n // 11
         have = inv(prec, n, b) - rest + slack
         for k in range(b, max(0, b - 200), -1):
             assert gemm(prec, n, b, b, k) <= have, (b, k)
