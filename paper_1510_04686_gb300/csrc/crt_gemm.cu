@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_st16(t_im + 2 * c0, im);
       }
       tmem_st_wait();
-      bool ok = !*abort_flag;
+      bool ok = __all_sync(0xffffffffu, !*abort_flag);
       int part = 0, mod = 0;
 #pragma unroll 1
       for (int step = 0; step < n_steps; ++step, ++use) {
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ++mod;
         }
         // u modulo p, packed as BF16 pairs (integers up to 256 are exact)
-        if (!ok || !mbar_wait(&accfull[0], use & 1, abort_flag)) {
+        if (!ok || !mbar_wait_warp(&accfull[0], use & 1, abort_flag)) {
           ok = false;
           break;
         }
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         release(0);
         // v modulo p, and the step's contribution to both fractions
-        if (!mbar_wait(&accfull[1], use & 1, abort_flag)) {
+        if (!mbar_wait_warp(&accfull[1], use & 1, abort_flag)) {
           ok = false;
           break;
         }

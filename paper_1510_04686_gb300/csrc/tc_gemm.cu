@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
     unsigned long long omax = 0ull;  // largest |Re|, |Im| this thread stores (rmax), as bits
     for (int acc = 0; acc < n_exec; ++acc) {
       const int buf = acc % kAccBufs;
-      if (!mbar_wait(&accfull[buf], (acc / kAccBufs) & 1, abort_flag)) break;
+      if (!mbar_wait_warp(&accfull[buf], (acc / kAccBufs) & 1, abort_flag)) break;
       tc_fence_after();
       const bool last = (acc == n_exec - 1);
       if (MINB == 1 && !last) {
