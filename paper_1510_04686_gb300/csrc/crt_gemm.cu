@@ -231,13 +231,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      // every load is waited for by the MMAs that read it; after a given-up wait nothing does, so
-      // loads in flight get time to land before this CTA's shared memory is released
-      if (*abort_flag) {
-        const unsigned long long t0 = gtimer();
-        while (gtimer() - t0 < 1000000ull) {
-        }
-      }
     }
   } else if (warp == kEpiWarps + 1) {
     // ---------------- MMA issuer 
@@ -535,6 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   __syncthreads();
+  land_in_flight(abort_flag);
   if (warp == kEpiWarps + 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),

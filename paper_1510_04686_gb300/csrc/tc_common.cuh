@@ -72,6 +72,16 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity,
                                                volatile int* abort_flag) {
   return __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag));
 }
+// Every load is waited for by the MMAs that read it, every MMA by the epilogue; after a given-up wait
+// nothing does.  All threads of a CTA call this, past a barrier behind the last wait (whichever role
+// gave up, and however early the producer was done), before shared or tensor memory is released.
+__device__ __forceinline__ void land_in_flight(volatile int* abort_flag) {
+  if (!*abort_flag) return;
+  const unsigned long long t0 = gtimer();
+  while (gtimer() - t0 < 1000000ull) {  // 1 ms
+  }
+  __syncwarp();
+}
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar,
                                             int x, int y, int z) {
   asm volatile(

@@ -554,6 +554,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
     }
   }
   __syncthreads();
+  land_in_flight(abort_flag);
   // the pair leaves together: no MMA of the even CTA may still reach the odd CTA's memory
   if constexpr (CG == 2) cluster_sync();
   if (warp == 9) {

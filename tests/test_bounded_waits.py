@@ -27,3 +27,14 @@ def test_a_warp_gives_up_as_a_whole(name):
     assert waits and min(waits) > roles.index("elect_one()")
     assert re.search(r"mbar_wait_warp\([^{]*\{\s*return __all_sync\(0xffffffffu, mbar_wait\(",
                      _code("tc_common.cuh"))
+
+
+@pytest.mark.parametrize("name", ["crt_gemm.cu", "tc_gemm.cu"])
+def test_copies_in_flight_land_before_memory_is_released(name):
+    """After the last wait of any role and a barrier, all threads give loads and MMAs in flight time to
+    land when a wait gave up; only then the CTA (or the pair) frees tensor memory and leaves."""
+    tail = _code(name).split("// ---------------- epilogue", 1)[1]
+    tail = tail[:tail.index("tcgen05.dealloc")]
+    last = tail[tail.rindex("mbar_wait"):]
+    assert re.search(r"__syncthreads\(\);\s*land_in_flight\(abort_flag\);", last)
+    assert "cluster_sync();" not in last.split("land_in_flight", 1)[0]
