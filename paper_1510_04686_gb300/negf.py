@@ -624,16 +624,20 @@ def solve_ragged(systems, opt: _Opt, outputs=("density", "current", "transmissio
     # the groups one after another; a thread per group lets their chains run side by side (the
     # library calls release the interpreter lock).  Four sizes of b = 200 ... 800, 4 points:
     # 330 -> 288 ms.
-    if concurrent and len(jobs) > 1 and opt.sr_host_check > 0:
-        library()  # loaded before the threads
-        with ThreadPoolExecutor(min(len(jobs), 16)) as ex:
-            for f in [ex.submit(solve, *job) for job in jobs]:
-                f.result()
-    else:
-        for job in jobs:
-            solve(*job)
-    for _, _, st in jobs:
-        cur.wait_stream(st)
+    try:
+        if concurrent and len(jobs) > 1 and opt.sr_host_check > 0:
+            library()  # loaded before the threads
+            with ThreadPoolExecutor(min(len(jobs), 16)) as ex:
+                for f in [ex.submit(solve, *job) for job in jobs]:
+                    f.result()
+        else:
+            for job in jobs:
+                solve(*job)
+    finally:
+        # also when a group fails: the others' kernels may still read the caller's tensors, whose
+        # memory is given out again in the order of `cur`
+        for _, _, st in jobs:
+            cur.wait_stream(st)
     return results
 
 
