@@ -81,8 +81,9 @@ def parse():
                     help="points per launch chain in the ragged workload (bounds each group's "
                          "workspace)")
     ap.add_argument("--tc-config", type=int, default=None,
-                    help="tensor-core GEMM configuration (default: autotuned per block size "
-                         "and batch for the rgf workload, the library default otherwise)")
+                    help="tensor-core GEMM configuration of calls of fewer than 12 points (default: "
+                         "autotuned per block size and batch for the rgf workload, the library "
+                         "default otherwise)")
     ap.add_argument("--scba-sigma", choices=["diag", "atom"], default="diag",
                     help="--workload scba: orbital-diagonal or atom-block (10 x 10) self-energies")
     ap.add_argument("--iface-orbitals", type=int, default=100,
@@ -567,7 +568,8 @@ def main():
         if args.tc_config is not None:
             tuned = negf.tc_config(args.tc_config)
         else:
-            # pick the tensor-core GEMM configuration for this block size and batch (untimed)
+            # pick the tensor-core GEMM configuration for this block size and batch (untimed; large
+            # batches have none to pick)
             from paper_1510_04686_gb300 import autotune
             tuned = autotune.tune_tc(WORK["b"], P)["config"]
     opt = negf.options(precision=prec, chunk=P)

@@ -75,13 +75,15 @@ typedef enum {
 /* Precision forms.  The mixed forms run every block GEMM on the tensor cores: each row of
  * op(A) and column of op(B) is scaled by a power of two and rounded once to fixed point (the
  * tiers are named 40, 48 and 56 bits), and the fixed-point product is formed exactly from BF16
- * operands; storage, pivoting, norms and reductions stay FP64.  Calls of 12 points (batch items)
- * or more form it modulo 10-15 small integers (residue products): a product's error is usually a
- * quarter of 2^-bits x |row of A| x |column of B| (2-norms) and stays below that unless its
- * roundings are equal term by term (lines of equal entries); in the 56-bit tier it is that of an
- * FP64 product.  A complex product issues 20 (40 bits), 24 (48 bits) or 28 (56 bits) real products
- * at 257-400 contracted terms.  Calls of fewer points cut the values into BF16 slices: the error is
- * about 2^-bits x K x max|row of A| x max|column of B|, for 60, 84 or 112 real products. */
+ * operands; storage, pivoting, norms and reductions stay FP64.  Calls of NEGF_RESIDUE_ITEMS points
+ * (batch items) or more form it modulo 10-15 small integers (residue products): a product's error
+ * is usually a quarter of 2^-bits x |row of A| x |column of B| (2-norms) and stays below that
+ * unless its roundings are equal term by term (lines of equal entries); in the 56-bit tier it is
+ * that of an FP64 product.  A complex product issues 20 (40 bits), 24 (48 bits) or 28 (56 bits)
+ * real products at 257-400 contracted terms.  Calls of fewer points cut the values into BF16
+ * slices: the error is about 2^-bits x K x max|row of A| x max|column of B|, for 60, 84 or 112
+ * real products. */
+#define NEGF_RESIDUE_ITEMS 12
 typedef enum {
   NEGF_PREC_FP64 = 0,     /* every block operation in FP64 on the CUDA cores (reference form) */
   NEGF_PREC_MIXED = 1,    /* tensor cores, 48-bit operand values (the default mixed form)     */
@@ -399,7 +401,7 @@ negf_status negf_zinv_batched_noalloc(int32_t n_batch, int32_t n, double* M, dou
                                       int32_t* status, void* stream);
 
 /* ---- tensor-core GEMM configuration (autotuning) ----------------------------------------
- * The mixed-precision GEMM of calls of fewer than 12 points or batch items (digit slices) has
+ * The mixed-precision GEMM of calls of fewer than NEGF_RESIDUE_ITEMS points (digit slices) has
  * negf_tc_config_count() kernel configurations, differing only in speed (that of larger calls
  * picks its tile by the product's size): configuration c uses the kernel shape c / 2 of
  *   (6 stages, 1 CTA, 1), (6, 1, 2), (6, 1, 3), (8 stages, CTA pair, 1), (8, 2, 2), (8, 2, 4),

@@ -1,8 +1,9 @@
 """Autotuner of the tensor-core GEMM configuration.
 
-Times every configuration of the mixed-precision batched complex GEMM (pipeline depth and K-part
-policy) on the block size and batch the sweeps use, picks the fastest, and caches the choice in
-``_tune/tc_<gpu>_b<b>_n<batch>.json`` beside the package so later runs reuse it.
+Times every configuration of the mixed-precision complex GEMM of small batches (pipeline depth and
+K-part policy) on the block size and batch the sweeps use, picks the fastest, and caches the choice in
+``_tune/tc_<gpu>_b<b>_n<batch>.json`` beside the package so later runs reuse it.  Batches of
+RESIDUE_ITEMS or more have no configuration to choose.
 """
 from __future__ import annotations
 
@@ -39,7 +40,11 @@ def load_cached(path: str):
 
 
 def tune_tc(b: int, batch: int, reps: int = 3, use_cache: bool = True) -> dict:
-    """Select and return the best configuration for b x b x b products in batches of `batch`."""
+    """Select and return the best configuration for b x b x b products in batches of `batch`.  A batch
+    whose products ignore the configuration leaves the present one, which later small calls use."""
+    if batch >= _n.RESIDUE_ITEMS:
+        return {"b": b, "batch": batch, "config": _n.tc_config(),
+                "n_configs": _n.tc_config_count(), "ms": {}}
     path = _key(b, batch)
     rec = load_cached(path) if use_cache else None
     if rec is not None:

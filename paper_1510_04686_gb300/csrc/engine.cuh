@@ -34,8 +34,7 @@ struct EngineWs {
 // bond current at an energy below the bias window is the small difference of two large terms, so
 // each form gives digits there that the arithmetic does not determine.  A batch of a dozen energies
 // or more has some inside the window, and is judged by the currents there.
-constexpr int kResidueItems = 12;
-inline bool residue_products(int n_items) { return n_items >= kResidueItems; }
+inline bool residue_products(int n_items) { return n_items >= NEGF_RESIDUE_ITEMS; }
 
 // Reserve the engine scratch for P concurrent b x b problems at `off` of `base` (base NULL:
 // only advance `off`).  precision: a negf_precision value, residues: the form of its products

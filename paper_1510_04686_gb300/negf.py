@@ -19,6 +19,7 @@ PREC_FP64 = 0
 PREC_MIXED = 1       # tensor cores, 48-bit operand values
 PREC_MIXED_40 = 2    # tensor cores, 40-bit operand values
 PREC_MIXED_56 = 3    # tensor cores, 56-bit operand values
+RESIDUE_ITEMS = 12   # points (batch items) from which mixed products ignore tc_config
 PREC_AUTO = -1       # lead_precision: FP64 for the FP64 form, else 56-bit (48 beyond b = 7008)
 SIGMA_ORBITAL_DIAG = 0  # scattering self-energies: one value per orbital
 SIGMA_ATOM_BLOCK = 1    # scattering self-energies: one atom_orbitals^2 block per atom
