@@ -115,8 +115,9 @@ struct Cfg {
   static constexpr int kBBox = NT * kKC * 2;
   static constexpr int kChunk = kABox + kBBox;
   // K chunks per stage.  Narrow tiles have little to do between a stage's barriers: two chunks per
-  // stage take 37 items of 333 x 217 x 591 from 490 to 473 us.  Wide ones need the stages: 64 items
-  // of 400^3 823 -> 850 us; nor do the correction sums leave the issuer waiting (603 -> 616 us).
+  // stage take 3.5 % less time for 37 items of 333 x 217 x 591 (418 us now).  Wide ones need the stages
+  // (64 items of 400^3, 731 us now, 3 % more with two chunks); nor do the correction sums leave the
+  // issuer waiting (2 % more).
   static constexpr int kPer = NT <= 64 && !HP ? 2 : 1;
   static constexpr int kStage = kPer * kChunk;
   static constexpr int kStages = std::min(10, (227 * 1024 - 1280) / kStage);

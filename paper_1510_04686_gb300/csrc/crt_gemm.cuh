@@ -8,6 +8,9 @@
 // sum of K products of them stays below 2^24 and is exact in the FP32 accumulator of the tensor
 // core (K is cut into parts where it is too long), and by Cauchy-Schwarz every result is below
 // P / 2, P the product of the moduli, so its residues determine it (Chinese remainder theorem).
+// (Products by residues of scaled integers are the method of Ozaki, Uchino and Imamura, "Ozaki scheme
+// II: a GEMM-oriented emulation of floating-point matrix multiplication using an integer modular
+// technique"; the form below is this library's own.)
 // The moduli split over the Gaussian integers, so a complex product takes two real products per
 // modulus (crt_plan.cuh): 24 of b x b x b for 48-bit values at b = 400, where fixed-point digit
 // products take 84 (21 digit pairs in the four-product real embedding).  The only rounding is

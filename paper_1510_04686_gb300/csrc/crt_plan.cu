@@ -17,10 +17,12 @@ using u128 = unsigned __int128;
 // Modulus classes.  Residues are at most (p + 1) / 2 in magnitude (exact in BF16 up to 256), so
 // a sum of K products stays below 2^24, exact in an FP32 accumulator, when
 // K ((p + 1) / 2)^2 <= 2^24.  Larger moduli carry more bits per product but fewer terms: each
-// class is the set of the largest usable moduli for the contraction lengths it names.
-constexpr int kMaxAlpha = 60;  // scaled values stay below 2^61 (64-bit fixed point, eight digits)
+// class is the set of the largest usable moduli for contractions (or parts of them) of up to the length
+// that it names.  The lengths rise by 1.25 from 256 to 1024; one of 320 is left out because it takes
+// as many moduli as 400 in every tier.
 constexpr int kClasses = 6;
 constexpr int kClassK[kClasses] = {256, 400, 512, 640, 800, 1024};
+constexpr int kMaxAlpha = 60;  // scaled values stay below 2^61 (64-bit fixed point, eight digits)
 
 struct Class {
   int count;

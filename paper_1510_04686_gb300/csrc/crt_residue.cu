@@ -193,8 +193,8 @@ __device__ __forceinline__ void write_planes(const ResidueConst& rc, const Coef&
 // plane and warp.  Bound by instruction issue, so that what counts is instructions per value: norms
 // take the FP32 value of a mantissa by a shift and a subtraction, sigma is a 64-bit integer
 // multiplication (as an FP64 one it held the two-lane FP64 pipe for a fifth of the kernel), and u and
-// v of a value are reduced as the neighbouring accumulators that they are.  A 64 x 400^3 product with
-// both its operands: 864 -> 817 us, the two conversions about 365 -> 320.
+// v of a value are reduced as the neighbouring accumulators that they are.  The two conversions of 64
+// products of 400^3 take 314 us (about 360 before these).
 template <int LINES, int NB>
 __global__ void __launch_bounds__(kThreads)
     k_residue_strip(const __grid_constant__ ResidueConst rc, int n, int alpha, unsigned long long sig,

@@ -27,13 +27,14 @@ struct EngineWs {
   bool residues;     // the form that tc was carved for
 };
 
-// Form of the tensor-core products of a call over n items (points, or matrices of a batch).
-// Residue products (crt_gemm.cuh) are the faster and the more accurate form at every size.  Calls
-// of few items keep digit-slice products (tc_gemm.cuh) and with them the results that they have
-// always given, because there the two forms can differ by more than rounding of the result: a
-// bond current at an energy below the bias window is the small difference of two large terms, so
-// each form gives digits there that the arithmetic does not determine.  A batch of a dozen energies
-// or more has some inside the window, and is judged by the currents there.
+// Form of the tensor-core products of a call over n items (points, or matrices of a batch): residue
+// products (crt_gemm.cuh) from NEGF_RESIDUE_ITEMS on, digit slices (tc_gemm.cuh) below.  The line is one
+// of results, not of speed or accuracy: calls of few items keep the digits that they gave before
+// residue products were there, and a point's last digits differ between calls on its two sides, by the
+// tier's error.  Residue products are the faster form below it too (us, digits / residues, 48 bits: 1
+// product of 100^3 87 / 71, 4 of 340^3 128 / 112, 8 of 600^3 574 / 311, 1 of 2400^3 2841 / 1192; 4
+// inverses of 340 1469 / 1426) and the nearer one to 64-bit results (sweeps of 1 to 8 points of b = 80
+// to 400: densities 5 to 50 times, currents 2 to 100 times).
 inline bool residue_products(int n_items) { return n_items >= NEGF_RESIDUE_ITEMS; }
 
 // Reserve the engine scratch for P concurrent b x b problems at `off` of `base` (base NULL:

@@ -3,11 +3,13 @@
 // for FP32 storage) and the pivot reciprocal in the storage precision (the FP32 form is refined
 // by Newton-Schulz steps afterwards).
 //
-// n <= small limit: one CTA per matrix, the whole matrix in shared memory.
-// larger n: blocked Gauss-Jordan.  A panel of nb columns is eliminated in shared memory, the
-// recorded row swaps are applied to the rest of the matrix and the remaining columns get the
-// rank-nb update  A[:, rest] += Panel * A[pivot rows, rest]  (pivot rows zeroed first), which is
-// a batched GEMM.  The column permutation is undone at the end.
+// Small n: one CTA per matrix, the whole matrix in shared memory.
+// Larger n: blocked Gauss-Jordan.  A panel of nb columns is eliminated, and the remaining columns get
+// the rank-nb update  A[:, rest] += Panel * A[pivot rows, rest]  (pivot rows zeroed first).  FP64 form:
+// the panel is eliminated in shared memory, the same kernel moves the exchanged rows of the whole
+// matrix, and the update is a batched product in place.  FP32 form: the panel is eliminated in registers
+// and no row is moved; the update reads the matrix through the panel's exchanges and writes it to a
+// second buffer.  The column permutation that the pivoting leaves is undone at the end.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -486,21 +488,6 @@ __global__ void __launch_bounds__(kThreads) k_gj_panel(int n, int k0, int w, int
   }
 }
 
-// FP32 form of the blocked elimination.  A panel is eliminated in registers, and the trailing
-// update reads the matrix through the panel's row exchanges and writes it to a second buffer, so no
-// pass over the matrix moves rows: src and dst alternate from panel to panel.
-//
-// Panel step: columns [k0, k0 + w) of src (w = W, the panel width, but for a matrix's LAST panel,
-// which may be narrower).  Thread (g, c) keeps rows g, g + kG, ... of column c in registers for all
-// steps; a step exchanges only the pivot column f, the two rows of the exchange and the pivot
-// through shared memory.  Writes the eliminated panel to U and to its columns of dst, the pivot
-// rows, and for every row the source row of its content after the panel's exchanges (cont).
-//
-// Bound by the chain of W steps (pivot search, exchange, update, a barrier between each) on one SM
-// per item: 65 us for 64 items of n = 400, W = 32, where a panel in shared memory on 256 threads
-// that also moved the rows of the whole matrix took 110 us.  512 threads: 1024 spend more on the
-// part of a step that every warp repeats, and a test per slot (instead of filler rows) parted the
-// slots' loads and took 140 us.
 // Pivot candidates.  hi + lo of mag2 is brought to h = RN(hi + lo) and the exact rest l, so that the
 // larger sum has the larger h, then the larger l; equal sums go to the lower row.  Keys order like
 // unsigned integers (a candidate's h key is at least 1), so a warp finds its winner with reductions
@@ -542,6 +529,21 @@ __device__ __forceinline__ cx<float> pivot_recip32(cx<float> a, int32_t* st) {
   return mkc<float>(__fmul_rn(ar, inv), __fmul_rn(-ai, inv));
 }
 
+// FP32 form of the blocked elimination.  A panel is eliminated in registers, and the trailing
+// update reads the matrix through the panel's row exchanges and writes it to a second buffer, so no
+// pass over the matrix moves rows: src and dst alternate from panel to panel.
+//
+// Panel step: columns [k0, k0 + w) of src (w = W, the panel width, but for a matrix's LAST panel,
+// which may be narrower).  Thread (g, c) keeps rows g, g + kG, ... of column c in registers for all
+// steps; a step exchanges only the pivot column f, the two rows of the exchange and the pivot
+// through shared memory.  Writes the eliminated panel to U and to its columns of dst, the pivot
+// rows, and for every row the source row of its content after the panel's exchanges (cont).
+//
+// Bound by the chain of W steps (pivot search, exchange, update, a barrier between each) on one SM
+// per item: 65 us for 64 items of n = 400, W = 32, where a panel in shared memory on 256 threads
+// that also moved the rows of the whole matrix took 110 us.  512 threads: 1024 spend more on the
+// part of a step that every warp repeats, and a test per slot (instead of filler rows) parted the
+// slots' loads and took 140 us.
 constexpr int kPanelThreads = 512, kPanelWarps = kPanelThreads / 32;
 template <int W, int NR, bool LAST>
 __global__ void __launch_bounds__(kPanelThreads)

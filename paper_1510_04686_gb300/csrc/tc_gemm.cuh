@@ -3,6 +3,10 @@
 //
 //   C = alpha op(A) op(B) + beta C + gamma D (+ I)       (complex128 in and out)
 //
+// (Error-free splitting of both operands is the method of Ozaki, Ogita, Oishi and Rump,
+// "Error-free transformations of matrix multiplication by using fast routines of matrix
+// multiplication and its applications".)
+//
 // Each operand row (A) / column (B) is scaled by a power of two, rounded once to a fixed-point
 // value of 40, 48 or 56 bits and cut into S slices of beta bits stored as BF16 (exact).  Slice
 // products are exact in BF16 x BF16 -> FP32 and, with beta and a split of K into parts chosen
